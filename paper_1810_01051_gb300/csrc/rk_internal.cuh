@@ -236,13 +236,17 @@ int launch_verify(const rk_table *t, const uint8_t *d_text, uint64_t n, const Ca
 int launch_sort(const rk_table *t, uint64_t n, uint64_t *d_keys, uint64_t capacity,
                 const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream);
 
-// Sort keys[0 .. d_info[0]) ascending over the 8-bit digits at the given bit
-// shifts (least significant first).  allow_fused: outputs of up to 32 tiles
-// per resident CTA may be sorted by one cooperative launch (every pass, grid
-// barriers between phases) instead of one look-back kernel per pass.
-int launch_sort_shifts(int sm_count, const uint32_t *shifts, uint32_t nshift, uint64_t *d_keys,
-                       uint64_t capacity, const uint64_t *d_info, void *d_ws, uint64_t ws_bytes,
-                       cudaStream_t stream, bool allow_fused);
+// The bits of a sort's keys that can be non-zero: lo_bits from bit 0 on and,
+// above them, hi_bits from bit hi_shift on.
+struct SortShape {
+    uint32_t lo_bits, hi_shift, hi_bits;
+};
+
+// Sort keys[0 .. d_info[0]) ascending, keys of the given shape: outputs of up
+// to 32 tiles per resident CTA in one cooperative launch, larger ones by one
+// look-back kernel per 8-bit digit.
+int launch_sort_shape(int sm_count, const SortShape &shape, uint64_t *d_keys, uint64_t capacity,
+                      const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream);
 
 uint64_t sort_workspace_bytes(uint64_t capacity);
 

@@ -1,14 +1,22 @@
 // A6: ascending order of the match keys key = (id << 40) | x, which is the
 // ascending (pattern id, offset) order the match list is defined in.
 //
-// Least-significant-digit radix sort over 8-bit digits.  Only the digits
-// that can be non-zero are sorted: those of the offset field (bits below
-// ceil(log2(n))) and of the id field (bits 40.. up to ceil(log2(k))).
+// Up to 32 tiles of 2048 keys per resident CTA: one cooperative launch that
+// sorts by cells (sort_cells below): the keys' bits that can be non-zero, as
+// one compact number, are cut into about one cell per key by their top bits;
+// the keys are counted and ranked per cell, scattered to their cell, and put
+// in order within it by comparison.  Keys crowded into few cells (more than
+// kCellMax in one) are sorted by the radix passes below instead, in the same
+// launch.
 //
+// Radix passes: least significant digit first over 8-bit digits, only those
+// that can be non-zero: those of the offset field (bits below ceil(log2(n)))
+// and of the id field (bits 40.. up to ceil(log2(k))).  Above the cooperative
+// launch's size:
 //   1. one histogram kernel reads the keys once and counts every pass's
 //      digits (the totals do not depend on the order), and clears the
 //      per-tile status words of the passes;
-//   2. one kernel per pass: each CTA takes the next tile of 4096 keys from a
+//   2. one kernel per pass: each CTA takes the next tile of 2048 keys from a
 //      counter, ranks its keys stably (ballot multisplit + per-warp digit counters),
 //      publishes its digit counts, adds up the counts of the tiles before it
 //      by looking back through their published words (decoupled look-back),
@@ -362,7 +370,241 @@ __device__ __forceinline__ void sort_one_tile(uint64_t *keys, uint64_t M, const 
     }
 }
 
-// Every pass in one cooperative launch, for outputs of a few thousand tiles.
+// ---- sort by cells -------------------------------------------------------
+// compact(key) has the key's order in shape.lo_bits + shape.hi_bits bits; a
+// cell holds the keys that share its top bits.  With about one cell per key
+// (2^cb in (M/2, M]) a cell of evenly spread keys holds a few, whatever the
+// number of digits: five grid barriers in place of three per digit, and each
+// key is read four times and written twice, mostly in L2.
+//
+// kCellMax: the comparisons within a cell cost its size squared; at 1024 keys
+// a cell they cost about what the radix passes do, which take over there.
+// Measured against the radix passes in one cooperative launch, as whole
+// searches: 10 M keys (4 GiB of bytes, 10,000 patterns) 4.38 -> 3.82 ms, 0.7 M
+// keys (64 MB of words) 270 -> 235 us, 78,000 keys (33 MB) 103 -> 77 us, 400
+// keys (1 MiB of DNA, one CTA) 37.9 -> 29.6 us.
+constexpr uint32_t kCellMax = 1024;
+constexpr uint32_t kOneCellBits = 12;  // cells of the one-CTA sort
+constexpr uint32_t kOneCellMax = 96;   // and the most keys it compares in one
+
+__device__ __forceinline__ uint64_t compact_key(uint64_t k, const SortShape &s) {
+    const uint64_t lo = s.lo_bits >= 64 ? k : k & ((1ull << s.lo_bits) - 1ull);
+    return s.hi_bits ? ((k >> s.hi_shift) << s.lo_bits) | lo : lo;
+}
+
+// Sum of v over the CTA, in every thread.
+__device__ __forceinline__ uint32_t cta_sum(uint32_t v, uint32_t *wsum, uint32_t lane,
+                                            uint32_t warp) {
+#pragma unroll
+    for (uint32_t d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    __syncthreads();
+    if (lane == 0) wsum[warp] = v;
+    __syncthreads();
+    uint32_t t = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < kWarps; ++w) t += wsum[w];
+    return t;
+}
+
+// Exclusive sum of v over the CTA's threads before this one; *total: of all.
+__device__ __forceinline__ uint32_t cta_excl(uint32_t v, uint32_t *wsum, uint32_t lane,
+                                             uint32_t warp, uint32_t *total) {
+    const uint32_t incl = warp_incl(v, lane);
+    __syncthreads();
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t before = 0, t = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < kWarps; ++w) {
+        before += w < warp ? wsum[w] : 0u;
+        t += wsum[w];
+    }
+    *total = t;
+    return before + incl - v;
+}
+
+// Up to kSortTile keys in one CTA, cells in shared memory.  Returns false,
+// with the keys untouched, when a cell holds too many.
+__device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const SortShape &shape,
+                                               uint64_t *sbuf, uint32_t *cell, uint32_t *wsum) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr uint32_t kCells = 1u << kOneCellBits, kPer = kCells / kThreads;
+    constexpr uint32_t kKeys = kSortTile / kThreads;
+    const uint32_t tb = shape.lo_bits + shape.hi_bits;
+    const uint32_t cs = tb > kOneCellBits ? tb - kOneCellBits : 0;
+    uint64_t key[kKeys];
+    uint32_t cr[kKeys];  // cell << 16 | rank in it
+#pragma unroll
+    for (uint32_t r = 0; r < kKeys; ++r) {
+        const uint32_t i = r * kThreads + tid;
+        key[r] = i < M ? __ldcg(keys + i) : 0;
+    }
+    for (uint32_t i = tid; i < kCells / 4; i += kThreads)
+        reinterpret_cast<uint4 *>(cell)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    bool crowded = false;
+#pragma unroll
+    for (uint32_t r = 0; r < kKeys; ++r)
+        if (r * kThreads + tid < M) {
+            const uint32_t c = (uint32_t)(compact_key(key[r], shape) >> cs);
+            const uint32_t k = atomicAdd(&cell[c], 1u);
+            crowded |= k >= kOneCellMax;
+            cr[r] = (c << 16) | k;
+        }
+    if (__syncthreads_or(crowded)) return false;
+    uint32_t v[kPer], sum = 0, total;
+#pragma unroll
+    for (uint32_t j = 0; j < kPer; ++j) {
+        v[j] = cell[tid * kPer + j];
+        sum += v[j];
+    }
+    uint32_t at = cta_excl(sum, wsum, lane, warp, &total);
+#pragma unroll
+    for (uint32_t j = 0; j < kPer; ++j) {
+        cell[tid * kPer + j] = at;
+        at += v[j];
+    }
+    if (tid == 0) cell[kCells] = M;
+    __syncthreads();
+#pragma unroll
+    for (uint32_t r = 0; r < kKeys; ++r)
+        if (r * kThreads + tid < M) sbuf[cell[cr[r] >> 16] + (cr[r] & 0xFFFFu)] = key[r];
+    __syncthreads();
+#pragma unroll
+    for (uint32_t r = 0; r < kKeys; ++r)
+        if (r * kThreads + tid < M) {
+            const uint32_t b = cell[cr[r] >> 16], e = cell[(cr[r] >> 16) + 1];
+            uint32_t less = 0;
+            for (uint32_t j = b; j < e; ++j) less += sbuf[j] < key[r];
+            keys[b + less] = key[r];
+        }
+    return true;
+}
+
+enum CellsResult { kCellsDone, kCellsCrowded, kCellsTimeout };
+
+// M keys over G CTAs of a cooperative launch.  cnt: 2^cb + 1 words, rank: M
+// half words, part: G words of workspace; flag and *bar start at zero.
+// kCellsCrowded (the same in every CTA): the keys are untouched.
+__device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp, uint64_t M,
+                                                  const SortShape &shape, uint32_t *cnt,
+                                                  uint16_t *rank, uint32_t *part, uint32_t cb,
+                                                  uint32_t *flag, unsigned int *bar, uint32_t G,
+                                                  unsigned int *passed, unsigned long long *info,
+                                                  uint32_t *wsum, int *s_ok) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t C = 1u << cb;
+    const uint32_t tb = shape.lo_bits + shape.hi_bits;
+    const uint32_t cs = tb > cb ? tb - cb : 0;
+    const uint64_t gid = blockIdx.x * (uint64_t)kThreads + tid, stride = (uint64_t)G * kThreads;
+    constexpr uint32_t kU = 8;  // keys in flight per thread
+
+    for (uint64_t i = gid; i < C / 4; i += stride)
+        __stcg(reinterpret_cast<uint4 *>(cnt) + i, make_uint4(0, 0, 0, 0));
+    if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
+
+    // count, and rank each key in its cell; the first key of every thread
+    // alone, so that crowded keys are noticed before they queue up on a cell
+    if (gid < M) {
+        const uint32_t c = (uint32_t)(compact_key(__ldcg(keys + gid), shape) >> cs);
+        const uint32_t r = atomicAdd(cnt + c, 1u);
+        rank[gid] = (uint16_t)r;
+        if (r >= kCellMax) *reinterpret_cast<volatile uint32_t *>(flag) = 1;
+    }
+    for (uint64_t i0 = gid + stride; i0 < M; i0 += kU * stride) {
+        if (*reinterpret_cast<volatile uint32_t *>(flag)) break;
+        uint64_t k[kU];
+        uint32_t r[kU];
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u) k[u] = i0 + u * stride < M ? __ldcg(keys + i0 + u * stride) : 0;
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u)
+            r[u] = i0 + u * stride < M
+                       ? atomicAdd(cnt + (uint32_t)(compact_key(k[u], shape) >> cs), 1u)
+                       : 0u;
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u)
+            if (i0 + u * stride < M) {
+                rank[i0 + u * stride] = (uint16_t)r[u];
+                if (r[u] >= kCellMax) *reinterpret_cast<volatile uint32_t *>(flag) = 1;
+            }
+    }
+    if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
+    if (__ldcg(flag)) return kCellsCrowded;
+
+    // exclusive sums of the counts: each CTA a run of cells, blocks of 1024
+    const uint32_t run = (C + G * 1024u - 1u) / (G * 1024u) * 1024u;
+    const uint32_t lo = min(C, blockIdx.x * run), hi = min(C, lo + run);
+    uint32_t mine = 0;
+    for (uint32_t i = lo + tid * 4; i < hi; i += kThreads * 4) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(cnt + i));
+        mine += v.x + v.y + v.z + v.w;
+    }
+    mine = cta_sum(mine, wsum, lane, warp);
+    if (tid == 0) part[blockIdx.x] = mine;
+    if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
+    uint32_t carry = 0;
+    for (uint32_t b = tid; b < blockIdx.x; b += kThreads) carry += __ldcg(part + b);
+    carry = cta_sum(carry, wsum, lane, warp);
+    for (uint32_t i0 = lo; i0 < hi; i0 += kThreads * 4) {
+        const uint32_t i = i0 + tid * 4;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (i < hi) v = __ldcg(reinterpret_cast<const uint4 *>(cnt + i));
+        uint32_t total;
+        const uint32_t at = carry + cta_excl(v.x + v.y + v.z + v.w, wsum, lane, warp, &total);
+        if (i < hi)
+            __stcg(reinterpret_cast<uint4 *>(cnt + i),
+                   make_uint4(at, at + v.x, at + v.x + v.y, at + v.x + v.y + v.z));
+        carry += total;
+    }
+    if (gid == 0) cnt[C] = (uint32_t)M;
+    if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
+
+    // scatter every key to its cell
+    for (uint64_t i0 = gid; i0 < M; i0 += kU * stride) {
+        uint64_t k[kU];
+        uint32_t at[kU];
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u) {
+            const uint64_t i = i0 + u * stride;
+            k[u] = i < M ? __ldcg(keys + i) : 0;
+            at[u] = i < M ? __ldcg(rank + i) : 0;
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u)
+            at[u] += __ldcg(cnt + (uint32_t)(compact_key(k[u], shape) >> cs));
+#pragma unroll
+        for (uint32_t u = 0; u < kU; ++u)
+            if (i0 + u * stride < M) tmp[at[u]] = k[u];
+    }
+    if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
+
+    // each key's place in its cell: the number of smaller keys there
+    constexpr uint32_t kV = 4;
+    for (uint64_t i0 = gid; i0 < M; i0 += kV * stride) {
+        uint64_t k[kV];
+        uint32_t b[kV], e[kV];
+#pragma unroll
+        for (uint32_t u = 0; u < kV; ++u) k[u] = i0 + u * stride < M ? __ldcg(tmp + i0 + u * stride) : 0;
+#pragma unroll
+        for (uint32_t u = 0; u < kV; ++u) {
+            const uint32_t c = (uint32_t)(compact_key(k[u], shape) >> cs);
+            b[u] = __ldcg(cnt + c);
+            e[u] = __ldcg(cnt + c + 1);
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < kV; ++u)
+            if (i0 + u * stride < M) {
+                uint32_t less = 0;
+                for (uint32_t j = b[u]; j < e[u]; ++j) less += tmp[j] < k[u];
+                keys[b[u] + less] = k[u];
+            }
+    }
+    return kCellsDone;
+}
+
+// The sort in one cooperative launch, for outputs of a few thousand tiles: by
+// cells, or by every radix pass when the keys are crowded.  For the passes
 // cnt holds, digit-major, the count of digit d among the keys of tile t at
 // [d * pitch + t].  Per pass:
 //   A  each CTA ranks its tile's keys stably (per-warp digit counters) and
@@ -379,7 +621,8 @@ __device__ __forceinline__ void sort_one_tile(uint64_t *keys, uint64_t M, const 
 // back from the second buffer.  CTAs beyond the tile count leave at once.
 __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
     uint64_t *keys, uint64_t *tmp, unsigned long long *info, uint64_t cap, Shifts sh,
-    uint32_t *cnt, uint32_t pitch, uint32_t *totals, unsigned int *bar) {
+    SortShape shape, uint32_t *cnt, uint32_t pitch, uint32_t *totals, unsigned int *bar,
+    uint32_t *flag) {
     uint64_t M;
     uint32_t T;
     if (!sort_count(info, cap, &M, &T)) return;
@@ -391,13 +634,25 @@ __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
     __shared__ int s_ok;
     if (T == 1) {
         __shared__ uint64_t sbuf[kSortTile];
-        sort_one_tile(keys, M, sh, sbuf, wcnt, dbase, wsum);
+        __shared__ __align__(16) uint32_t cell[(1u << kOneCellBits) + 4];
+        if (!sort_one_cells(keys, (uint32_t)M, shape, sbuf, cell, wsum))
+            sort_one_tile(keys, M, sh, sbuf, wcnt, dbase, wsum);
         return;
+    }
+    unsigned int passed = 0;
+    {
+        // 2^cb <= M cells (words), then M ranks (half words), then a word per
+        // CTA: at most 12 of the 16 KiB of look-back words that a tile has
+        const uint32_t cb = 31u - __clz((uint32_t)M);
+        uint16_t *rank = reinterpret_cast<uint16_t *>(cnt + (1u << cb) + 4);
+        uint32_t *part = reinterpret_cast<uint32_t *>(rank + (M + 1) / 2 * 2);
+        const CellsResult r = sort_cells(keys, tmp, M, shape, cnt, rank, part, cb, flag, bar, G,
+                                         &passed, info, wsum, &s_ok);
+        if (r != kCellsCrowded) return;
     }
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     const bool one = T <= G;  // one tile per CTA: state kept from A to C
-    unsigned int passed = 0;
     uint64_t key[kPerWarp / 32];
     uint32_t rank[kPerWarp / 32];
     for (uint32_t p = 0; p < sh.n; ++p) {
@@ -545,32 +800,37 @@ constexpr uint64_t kFusedTilesPerCta = 32;
 
 // CTAs of the fused sort for an output of `capacity` keys (0: the look-back
 // kernels are used instead).
-uint32_t fused_ctas(int sm_count, uint64_t capacity, bool allow_fused) {
-    const uint32_t gmax = allow_fused ? fused_grid(sm_count) : 0;
+uint32_t fused_ctas(int sm_count, uint64_t capacity) {
+    const uint32_t gmax = fused_grid(sm_count);
     const uint64_t tiles = sort_ws_layout(capacity).tiles;
     if (!gmax || tiles > kFusedTilesPerCta * gmax) return 0;
     return (uint32_t)std::min<uint64_t>(tiles, gmax);
 }
 
-// The digit shifts of a plain search's keys: the offset field's bits below
-// ceil(log2(n)), then the id field's bits up to ceil(log2(k)).
-uint32_t plain_shifts(uint64_t n, uint32_t k, uint32_t *shifts) {
-    uint32_t ns = 0;
-    const uint32_t ob = bits_for(n - 1), pb = bits_for(k - 1);
-    for (uint32_t s = 0; s < ob; s += 8) shifts[ns++] = s;
-    for (uint32_t s = 0; s < pb; s += 8) shifts[ns++] = RK_KEY_OFFSET_BITS + s;
-    return ns;
+// The fields of a plain search's keys that can be non-zero.
+SortShape plain_shape(uint64_t n, uint32_t k) {
+    return SortShape{bits_for(n - 1), RK_KEY_OFFSET_BITS, bits_for(k - 1)};
+}
+
+// The radix passes' digit shifts for a key shape, least significant first.
+Shifts shifts_of(const SortShape &shape) {
+    Shifts sh{};
+    for (uint32_t s = 0; s < shape.lo_bits; s += 8) sh.s[sh.n++] = s;
+    for (uint32_t s = 0; s < shape.hi_bits; s += 8) sh.s[sh.n++] = shape.hi_shift + s;
+    return sh;
 }
 
 }  // namespace
 
 uint64_t sort_workspace_bytes(uint64_t capacity) { return sort_ws_bytes(capacity); }
 
-int launch_sort_shifts(int sm_count, const uint32_t *shifts, uint32_t nshift, uint64_t *d_keys,
-                       uint64_t capacity, const uint64_t *d_info, void *d_ws, uint64_t ws_bytes,
-                       cudaStream_t stream, bool allow_fused) {
-    if (capacity < 2 || nshift == 0) return RK_OK;
-    if (nshift > kMaxSortPasses || ws_bytes < sort_ws_bytes(capacity)) return RK_EINVAL;
+int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
+                      uint64_t capacity, const uint64_t *d_info, void *d_ws, uint64_t ws_bytes,
+                      cudaStream_t stream) {
+    SortShape shape = shape_in;
+    Shifts sh = shifts_of(shape);
+    if (capacity < 2 || sh.n == 0) return RK_OK;
+    if (ws_bytes < sort_ws_bytes(capacity)) return RK_EINVAL;
     const SortWsLayout L = sort_ws_layout(capacity);
     uint8_t *ws = reinterpret_cast<uint8_t *>(d_ws);
     uint64_t *tmp = reinterpret_cast<uint64_t *>(ws + L.tmp_off);
@@ -579,19 +839,20 @@ int launch_sort_shifts(int sm_count, const uint32_t *shifts, uint32_t nshift, ui
     uint64_t *status = reinterpret_cast<uint64_t *>(ws + L.status_off);
     unsigned long long *info =
         reinterpret_cast<unsigned long long *>(const_cast<uint64_t *>(d_info));
-    Shifts sh{};
-    for (uint32_t i = 0; i < nshift; ++i) sh.s[sh.n++] = shifts[i];
 
-    if (cudaMemsetAsync(ws + L.ctrl_off, 0, L.status_off - L.ctrl_off, stream) != cudaSuccess)
-        return RK_ECUDA;
-    // up to kFusedTilesPerCta tiles per CTA: every pass in one cooperative launch
-    if (const uint32_t g = fused_ctas(sm_count, capacity, allow_fused)) {
-        // digit-major counts, 256 x tiles (in the look-back words' space)
+    // up to kFusedTilesPerCta tiles per CTA: one cooperative launch
+    if (const uint32_t g = fused_ctas(sm_count, capacity)) {
+        // its barrier and flag are the control words; cell counts and ranks,
+        // or digit-major counts (256 x tiles), go to the look-back words' space
+        if (cudaMemsetAsync(counters, 0, L.ghist_off - L.ctrl_off, stream) != cudaSuccess)
+            return RK_ECUDA;
         uint32_t *cnt = reinterpret_cast<uint32_t *>(status);
         uint32_t pitch = (uint32_t)L.tiles;
         uint32_t *totals = ghist;
         unsigned int *bar = counters + 32;
-        void *args[] = {&d_keys, &tmp, &info, &capacity, &sh, &cnt, &pitch, &totals, &bar};
+        uint32_t *flag = counters;
+        void *args[] = {&d_keys, &tmp, &info,   &capacity, &sh,  &shape,
+                        &cnt,    &pitch, &totals, &bar,      &flag};
         if (cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(rk_sort_fused_kernel), g,
                                         kThreads, args, 0, stream) != cudaSuccess) {
             cudaGetLastError();
@@ -599,6 +860,8 @@ int launch_sort_shifts(int sm_count, const uint32_t *shifts, uint32_t nshift, ui
         }
         return RK_OK;
     }
+    if (cudaMemsetAsync(ws + L.ctrl_off, 0, L.status_off - L.ctrl_off, stream) != cudaSuccess)
+        return RK_ECUDA;
     // histogram grid: about one CTA per 4096 keys of the capacity, at most 4 per SM
     const uint32_t grid =
         (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)sm_count * 4,
@@ -622,18 +885,15 @@ int launch_sort_shifts(int sm_count, const uint32_t *shifts, uint32_t nshift, ui
 int launch_sort(const rk_table *t, uint64_t n, uint64_t *d_keys, uint64_t capacity,
                 const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream) {
     if (n == 0 || t->dev.n_patterns == 0) return RK_OK;
-    uint32_t shifts[kMaxSortPasses];
-    const uint32_t ns = plain_shifts(n, t->dev.n_patterns, shifts);
-    return launch_sort_shifts(t->sm_count, shifts, ns, d_keys, capacity, d_info, d_ws, ws_bytes,
-                              stream, true);
+    return launch_sort_shape(t->sm_count, plain_shape(n, t->dev.n_patterns), d_keys, capacity,
+                             d_info, d_ws, ws_bytes, stream);
 }
 
 uint32_t sort_launches(const rk_table *t, uint64_t n, uint64_t capacity) {
     if (n == 0 || t->dev.n_patterns == 0 || capacity < 2) return 0;
-    uint32_t shifts[kMaxSortPasses];
-    const uint32_t ns = plain_shifts(n, t->dev.n_patterns, shifts);
+    const uint32_t ns = shifts_of(plain_shape(n, t->dev.n_patterns)).n;
     if (ns == 0) return 0;
-    if (fused_ctas(t->sm_count, capacity, true)) return 1;
+    if (fused_ctas(t->sm_count, capacity)) return 1;
     return 1 + ns + (ns & 1);  // histogram, one kernel per pass, copy back
 }
 
