@@ -276,9 +276,10 @@ uint32_t bits_for(uint64_t max_value) {
 }
 
 template <int MODE, bool Q4, int MAXW, bool S2S>
-cudaError_t set_attr(uint32_t smem) {
-    return cudaFuncSetAttribute(rk_batch_tiles_kernel<MODE, Q4, MAXW, S2S>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t set_attr() {
+    static std::atomic<uint64_t> done{0};
+    return allow_smem(reinterpret_cast<const void *>(rk_batch_tiles_kernel<MODE, Q4, MAXW, S2S>),
+                      &done);
 }
 
 template <int MODE, bool Q4, int MAXW, bool S2S>
@@ -291,7 +292,7 @@ template <int MODE, bool Q4>
 cudaError_t dispatch_w(bool attr, const BatchParams &p, uint32_t grid, uint32_t smem,
                        cudaStream_t st) {
 #define RK_B(MW, S)                                                    \
-    return attr ? set_attr<MODE, Q4, MW, S>(smem) : launch_b<MODE, Q4, MW, S>(p, grid, smem, st)
+    return attr ? set_attr<MODE, Q4, MW, S>() : launch_b<MODE, Q4, MW, S>(p, grid, smem, st)
     if (p.warps <= 8) {
         if (p.s2slot) { RK_B(8, true); } else { RK_B(8, false); }
     }

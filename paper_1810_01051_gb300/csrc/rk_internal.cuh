@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -254,6 +255,13 @@ uint64_t sort_workspace_bytes(uint64_t capacity);
 uint32_t sort_launches(const rk_table *t, uint64_t n, uint64_t capacity);
 
 int check_device(const rk_table *t);
+
+// Allow a kernel the most dynamic shared memory a launch of this library uses
+// (the opt-in size per block less 1 KiB), once per device; `done` is the
+// kernel's own, one bit per device.  The limit belongs to the function, not to
+// the calling thread: one set per launch size would be lowered by another
+// thread's smaller table between this thread's check and its launch.
+cudaError_t allow_smem(const void *fn, std::atomic<uint64_t> *done);
 
 }  // namespace rk
 

@@ -55,6 +55,19 @@ int launch_scan(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t x
                             kWaitTimeoutNs, false, cand);
 }
 
+cudaError_t allow_smem(const void *fn, std::atomic<uint64_t> *done) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (done->load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - 1024);
+    if (e == cudaSuccess) done->fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
+
 bool can_defer(const rk_table *t) {
     return t->dev.filter_mode != kFilterNone &&
            t->dev.gram_bits <= kCandClassShift - kCandSlotShift;

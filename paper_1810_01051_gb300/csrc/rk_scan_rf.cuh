@@ -499,19 +499,9 @@ cudaError_t launch_rf_w(const ScanParams &p, uint32_t grid, uint32_t threads, ui
                         cudaStream_t st) {
     auto fn = p.s2_smem ? rk_scan_rf_kernel<KIND, MAXW, true, DEFER>
                         : rk_scan_rf_kernel<KIND, MAXW, false, DEFER>;
-    // raise the dynamic shared-memory limit once per device and size
-    static thread_local int seen_dev[2] = {-1, -1};
-    static thread_local uint32_t seen_smem[2] = {0, 0};
-    const int slot = p.s2_smem ? 1 : 0;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (seen_dev[slot] != dev || seen_smem[slot] < smem) {
-        cudaError_t e =
-            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        seen_dev[slot] = dev;
-        seen_smem[slot] = smem;
-    }
+    static std::atomic<uint64_t> done[2] = {};
+    const cudaError_t e = allow_smem(reinterpret_cast<const void *>(fn), &done[p.s2_smem ? 1 : 0]);
+    if (e != cudaSuccess) return e;
     fn<<<grid, threads, smem, st>>>(p);
     return cudaGetLastError();
 }
