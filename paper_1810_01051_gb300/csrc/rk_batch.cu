@@ -213,11 +213,12 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
             C.pid_shift = P.ob;
             C.q = tab->q;
             C.gram_bits = tab->gram_bits;
+            C.gram_mult = tab->gram_mult;
             C.base_log2 = tab->base_log2;
             C.n_lengths = tab->n_lengths;
             fmask = tab->filter_mask;
             qmask = C.q == 4 ? 0xFFFFFFFFu : (1u << (8u * C.q)) - 1u;
-            if (!S2S) C.s2 = make_s2(*tab, tab->s2_base);
+            if (!S2S) C.s2 = make_s2<MODE == kFilterNone>(*tab, tab->s2_base);
         }
         if (S2S) {
             // the survivor tables sit in this stage's slot (placed there by
@@ -225,14 +226,14 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
             DevTable tt;
             tt.s2_base = tab->s2_base;
             tt.grams = tab->grams;
-            tt.gram_lens = tab->gram_lens;
+            tt.gram_runs = tab->gram_runs;
             tt.group_hdr = tab->group_hdr;
             tt.slots = tab->slots;
             tt.group_pids = tab->group_pids;
             tt.pbytes = tab->pbytes;
             tt.poff = tab->poff;
             tt.lengths = tab->lengths;
-            C.s2 = make_s2(tt, sb + lay.s2_in_stage);
+            C.s2 = make_s2<MODE == kFilterNone>(tt, sb + lay.s2_in_stage);
         }
         const uint8_t *buf = sb + lay.text_in_stage;
         const uint64_t u0 = (uint64_t)d.y * P.tile;

@@ -15,7 +15,8 @@ namespace rk {
 // Mersenne prime modulus of the Rabin hash: p = 2^61 - 1.
 constexpr uint64_t kP61 = (1ull << 61) - 1;
 
-// Multipliers of the multiplicative hashes that place keys in tables.
+// Multipliers of the multiplicative hashes that place keys in tables (kGramMult:
+// the sample map, and the first one tried for the prefix map).
 constexpr uint32_t kFilterMult = 0x85EBCA77u;
 constexpr uint32_t kGramMult = 0x9E3779B1u;
 constexpr uint64_t kGroupMult = 0x9E3779B97F4A7C15ull;
@@ -32,11 +33,13 @@ struct GroupSlot {
 };
 
 // One slot of the prefix map: a q-byte pattern prefix (little-endian value),
-// the run [first, first+count) of distinct pattern lengths in gram_lens, and
-// `ext`, a 32-bit fingerprint set of the next four bytes (bytes q..q+3) of
-// the patterns with this prefix that are at least q + 4 bytes long; bit 31 of
-// `count` (kGramShort) marks a prefix that also has a shorter pattern.
-struct GramSlot {
+// its `count` runs (one per distinct length of the patterns that start with
+// it, lengths ascending), and `ext`, a 32-bit fingerprint set of the next four
+// bytes (bytes q..q+3) of the patterns with this prefix that are at least
+// q + 4 bytes long; bit 31 of `count` (kGramShort) marks a prefix that also has
+// a shorter pattern.  Run 0 of slot i is gram_runs[i], so it can be read with
+// the slot; run j > 0 is gram_runs[first + j].
+struct alignas(16) GramSlot {
     uint32_t key;
     uint32_t first;
     uint32_t count;  // 0 = empty slot; bit 31: some length is below q + 4
@@ -44,12 +47,28 @@ struct GramSlot {
 };
 constexpr uint32_t kGramShort = 1u << 31;
 
-// One slot of the sample map: a 4-byte gram (little-endian) and the set of
-// offsets j (bit j, j < 4) at which it starts in some pattern; mask 0 = empty.
-struct SampSlot {
+// The patterns of one prefix and length: a single one (id and offset of its
+// bytes in pbytes, in 8-byte units: a window is compared with it at once), or
+// several (pid == kManyPids: found by the window's hash in the length's table).
+struct alignas(16) LenRun {
+    uint32_t len;
+    uint32_t pid;
+    uint32_t off;
+    uint32_t pad;
+};
+constexpr uint32_t kManyPids = 0xFFFFFFFFu;
+
+// One slot of the sample map: a 4-byte gram (little-endian), the set of
+// offsets j (bit j, j < 4) at which it starts in some pattern (0 = empty), and,
+// when it occurs at one offset and after one prefix only, that prefix's slot
+// of the prefix map (else kNoSlot).
+struct alignas(16) SampSlot {
     uint32_t key;
     uint32_t mask;
+    uint32_t gi;
+    uint32_t pad;
 };
+constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 
 // Bit of `ext` for four bytes read as a little-endian word.
 __host__ __device__ __forceinline__ uint32_t ext_bit(uint32_t w) {
@@ -66,8 +85,8 @@ struct DevTable {
     uint32_t q;               // stage-1 key length in bytes, 1..4 (little-endian prefix)
 
     const GramSlot *grams;    // prefix map, 2^gram_bits slots
-    uint32_t gram_bits;
-    const uint32_t *gram_lens;
+    uint32_t gram_bits, gram_mult;  // a key's home slot: (key * gram_mult) >> (32 - gram_bits)
+    const LenRun *gram_runs;
 
     const uint2 *group_hdr;   // per length L = 0..lmax: {first slot, log2 slots}; .y == 0: none
     const GroupSlot *slots;
@@ -114,9 +133,10 @@ struct DevTable {
     uint32_t lmin, lmax;
     uint32_t base_log2;
 
-    // Every array above except the bit set lies in [s2_base, s2_base +
-    // s2_bytes): the survivor-stage tables, which the scan kernel may copy to
-    // shared memory as one block.
+    // The prefix map, its runs, the pattern bytes and the sample map lie in
+    // [s2_base, s2_base + s2_bytes): the survivor-stage tables, which the scan
+    // kernel may copy to shared memory as one block.  Without a prefilter
+    // (kFilterNone) the block goes on to the lengths' hash tables.
     const uint8_t *s2_base;
     uint32_t s2_bytes;
 };
@@ -187,7 +207,7 @@ namespace rk {
 // offsets of its parts; `meta` holds the device view's non-pointer fields.
 struct TableBlob {
     std::vector<uint8_t> bytes;
-    size_t o_filter = 0, o_grams = 0, o_glens = 0, o_ghdr = 0, o_slots = 0, o_gpids = 0,
+    size_t o_filter = 0, o_grams = 0, o_runs = 0, o_ghdr = 0, o_slots = 0, o_gpids = 0,
            o_pbytes = 0, o_poff = 0, o_plen = 0, o_lens = 0, o_sfilter = 0, o_smap = 0,
            o_rfilter = 0;
     DevTable meta{};

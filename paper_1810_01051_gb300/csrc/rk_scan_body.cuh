@@ -1,8 +1,10 @@
 // Device code that processes one staged text tile: the per-window prefilter
 // (stage 1), the per-warp survivor queue, and for survivors the Rabin hash
 // mod 2^61 - 1 at each candidate pattern length (A2), the probe of that
-// length's table (A3), the byte comparison (A4) and buffered emission (A5).
-// Shared by the single-text scan kernel and the batch kernel.
+// length's table (A3), the byte comparison (A4) and buffered emission (A5).  A
+// prefix and length that one pattern has alone goes straight to A4.
+// Shared by the single-text scan kernels, the verification kernel and the batch
+// kernel.
 #pragma once
 
 #include "rk_internal.cuh"
@@ -97,7 +99,7 @@ __device__ __forceinline__ bool verify(const Src &src, Pos pos, const uint8_t *p
 // Survivor-stage tables, as pointers into shared or global memory.
 struct S2 {
     const GramSlot *grams;
-    const uint32_t *gram_lens;
+    const LenRun *gram_runs;
     const uint2 *group_hdr;
     const GroupSlot *slots;
     const uint32_t *group_pids;
@@ -112,19 +114,21 @@ __device__ __forceinline__ const T *rebase(const T *p, const uint8_t *from, cons
     return reinterpret_cast<const T *>(to + (reinterpret_cast<const uint8_t *>(p) - from));
 }
 
-// The survivor tables of `T`, moved to `to` when they were copied there.
+// The survivor tables of `T`, moved to `to` when they were copied there (ALL:
+// the lengths' hash tables with them, as without a prefilter).
+template <bool ALL>
 __device__ __forceinline__ S2 make_s2(const DevTable &T, const uint8_t *to) {
     S2 s;
-    const uint8_t *from = T.s2_base;
+    const uint8_t *from = T.s2_base, *all = ALL ? to : from;
     s.grams = rebase(T.grams, from, to);
-    s.gram_lens = rebase(T.gram_lens, from, to);
-    s.group_hdr = rebase(T.group_hdr, from, to);
-    s.slots = rebase(T.slots, from, to);
-    s.group_pids = rebase(T.group_pids, from, to);
+    s.gram_runs = rebase(T.gram_runs, from, to);
     s.pbytes = rebase(T.pbytes, from, to);
-    s.poff = rebase(T.poff, from, to);
-    s.lengths = rebase(T.lengths, from, to);
     s.smap = rebase(T.smap, from, to);
+    s.group_hdr = rebase(T.group_hdr, from, all);
+    s.slots = rebase(T.slots, from, all);
+    s.group_pids = rebase(T.group_pids, from, all);
+    s.poff = rebase(T.poff, from, all);
+    s.lengths = rebase(T.lengths, from, all);
     return s;
 }
 
@@ -136,7 +140,7 @@ struct WinCtx {
     uint64_t n;           // text length
     uint64_t key_prefix;  // or-ed into every key
     uint32_t pid_shift;   // bit position of the pattern id in a key
-    uint32_t q, gram_bits, base_log2, n_lengths;
+    uint32_t q, gram_bits, gram_mult, base_log2, n_lengths;
     uint32_t smap_bits;   // sampled tables: sample map size (log2 slots)
 };
 
@@ -164,10 +168,16 @@ __device__ __forceinline__ void emit_global(const WarpCtx &w, uint64_t key) {
     if (g < w.capacity) w.keys[g] = key;
 }
 
+// A shared word that the warp's lanes add to, read as one value by all of them
+// (each lane's own read could see another lane's next addition).
+__device__ __forceinline__ uint32_t warp_read(const uint32_t *p) {
+    return __shfl_sync(0xffffffffu, *reinterpret_cast<const volatile uint32_t *>(p), 0);
+}
+
 // Warp-converged: move the buffered matches to the output with one atomic.
 __device__ __forceinline__ void flush(const WarpCtx &w, uint32_t lane) {
     __syncwarp();
-    uint32_t cnt = min(*reinterpret_cast<volatile uint32_t *>(w.mcount), kMatchCap);
+    uint32_t cnt = min(warp_read(w.mcount), kMatchCap);
     if (cnt) {
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(&w.info[0], (unsigned long long)cnt);
@@ -208,43 +218,14 @@ __device__ __forceinline__ void probe_length(const WinCtx &C, const WarpCtx &w, 
     }
 }
 
-// Stage 2 for one window at buffer position pos of the tile starting at u0.
-template <int MODE>
-__device__ __forceinline__ void process_window(const WinCtx &C, const WarpCtx &w,
-                                               const uint8_t *buf, uint32_t pos, uint64_t u0) {
-    const uint64_t ua = u0 + pos;
-    if (ua < C.lo || ua >= C.hi) return;
-    const uint64_t x = ua - C.mis;
-    if (MODE == kFilterNone) {
-        for (uint32_t i = 0; i < C.n_lengths; ++i) {
-            const uint32_t L = C.s2.lengths[i];
-            if (x + L > C.n) break;
-            probe_length(C, w, buf, pos, x, L);
-        }
-        return;
-    }
-    const uint64_t v = ld8(buf, pos);  // window bytes 0..7, little-endian
-    const uint32_t key = C.q == 4 ? (uint32_t)v : (uint32_t)v & ((1u << (8u * C.q)) - 1u);
-    const uint32_t gmask = (1u << C.gram_bits) - 1u;
-    uint32_t idx = (key * kGramMult) >> (32u - C.gram_bits);
-    for (;;) {
-        const GramSlot g = C.s2.grams[idx];
-        if (g.count == 0) return;  // a false positive of the bit set
-        if (g.key == key) {
-            // patterns of length >= q + 4 need bytes q..q+3 in the fingerprint set
-            const bool ext_ok = (g.ext >> ext_bit((uint32_t)(v >> (8u * C.q)))) & 1u;
-            if (!ext_ok && !(g.count & kGramShort)) return;  // every length is >= q + 4
-            const uint32_t cnt = g.count & ~kGramShort;
-            for (uint32_t j = 0; j < cnt; ++j) {
-                const uint32_t L = C.s2.gram_lens[g.first + j];
-                if (x + L > C.n) break;  // lengths ascend
-                if (L >= C.q + 4 && !ext_ok) break;
-                probe_length(C, w, buf, pos, x, L);
-            }
-            return;
-        }
-        idx = (idx + 1) & gmask;
-    }
+// The pattern of a run that names one against the window at pos (text offset x).
+template <bool DIRECT, class Src, class Pos>
+__device__ __forceinline__ void compare_one(const WinCtx &C, const WarpCtx &w, const Src &src,
+                                            Pos pos, uint64_t x, const LenRun &r) {
+    if (!verify(src, pos, C.s2.pbytes + 8ull * r.off, r.len)) return;
+    const uint64_t key = C.key_prefix | ((uint64_t)r.pid << C.pid_shift) | x;
+    if (DIRECT) emit_global(w, key);
+    else emit(w, key);
 }
 
 // Deferred verification (filtered modes).  Stage 2a below only finds the
@@ -286,7 +267,7 @@ constexpr uint32_t kCandBuf = kMatchCap / 2;     // 16-byte candidates in a warp
 __device__ __forceinline__ int gram_lookup_v8(const WinCtx &C, uint64_t v) {
     const uint32_t key = C.q == 4 ? (uint32_t)v : (uint32_t)v & ((1u << (8u * C.q)) - 1u);
     const uint32_t gmask = (1u << C.gram_bits) - 1u;
-    uint32_t idx = (key * kGramMult) >> (32u - C.gram_bits);
+    uint32_t idx = (key * C.gram_mult) >> (32u - C.gram_bits);
     for (;;) {
         const GramSlot g = C.s2.grams[idx];
         if (g.count == 0) return -1;
@@ -306,8 +287,10 @@ __device__ __forceinline__ int gram_lookup(const WinCtx &C, const Src &src, Pos 
     return gram_lookup_v8(C, v);
 }
 
-// Probe every length of prefix-map slot gi that applies to the window at pos
-// (text offset x): A2 hash, A3 probe, A4 verify, A5 emit.
+// Complete the candidate of prefix-map slot gi at window pos (text offset x):
+// every run that applies, by one comparison (A4), or, where several patterns
+// share prefix and length, by hash, probe and comparisons (A2, A3, A4); matches
+// emitted (A5).
 template <bool DIRECT = false, class Src, class Pos>
 __device__ __forceinline__ void probe_slot(const WinCtx &C, const WarpCtx &w, const Src &src,
                                            Pos pos, uint64_t x, uint32_t gi,
@@ -316,11 +299,35 @@ __device__ __forceinline__ void probe_slot(const WinCtx &C, const WarpCtx &w, co
     const bool ext_ok = (g.ext >> ext_bit((uint32_t)(ld8(src, pos) >> (8u * C.q)))) & 1u;
     const uint32_t cnt = g.count & ~kGramShort;
     for (uint32_t j = 0; j < cnt; ++j) {
-        const uint32_t L = C.s2.gram_lens[g.first + j];
-        if (x + L > C.n) break;  // lengths ascend
-        if (L >= C.q + 4 && !ext_ok) break;
-        if (len_in_class(L, cls)) probe_length<DIRECT>(C, w, src, pos, x, L);
+        const LenRun r = C.s2.gram_runs[g.first + j];
+        if (x + r.len > C.n) break;  // lengths ascend
+        if (r.len >= C.q + 4 && !ext_ok) break;
+        if (!len_in_class(r.len, cls)) continue;
+        if (r.pid != kManyPids) compare_one<DIRECT>(C, w, src, pos, x, r);
+        else probe_length<DIRECT>(C, w, src, pos, x, r.len);
     }
+}
+
+// Every stage after the first for one window at buffer position pos of the
+// tile starting at u0: with a prefilter the exact prefix and its runs, without
+// one every length by hash.
+template <int MODE>
+__device__ __forceinline__ void process_window(const WinCtx &C, const WarpCtx &w,
+                                               const uint8_t *buf, uint32_t pos, uint64_t u0) {
+    const uint64_t ua = u0 + pos;
+    if (ua < C.lo || ua >= C.hi) return;
+    const uint64_t x = ua - C.mis;
+    if (MODE == kFilterNone) {
+        for (uint32_t i = 0; i < C.n_lengths; ++i) {
+            const uint32_t L = C.s2.lengths[i];
+            if (x + L > C.n) break;
+            probe_length(C, w, buf, pos, x, L);
+        }
+        return;
+    }
+    uint64_t v8;
+    const int gi = gram_lookup(C, buf, pos, &v8);
+    if (gi >= 0) probe_slot(C, w, buf, pos, x, (uint32_t)gi);
 }
 
 // A candidate for which the list has no room is probed at once, with its
@@ -332,16 +339,23 @@ __device__ __forceinline__ void cand_overflow(const WinCtx &C, const WarpCtx &w,
     probe_slot<true>(C, w, buf, (uint32_t)(x + C.mis - u0), x, cand_slot(e), cand_class(e));
 }
 
-// Stage 2a for the window at pos of the tile at u0; a candidate is queued in
+// Stage 2a for the window at pos of the tile at u0 (known: its prefix-map slot,
+// when the sample map names it); a candidate is queued in
 // the warp's buffer (w.mbuf as kCandBuf 16-byte entries), or offered to the
 // list when that is full.
 __device__ __forceinline__ void cand_window(const WinCtx &C, const WarpCtx &w, const CandList &cc,
-                                            const uint8_t *buf, uint32_t pos, uint64_t u0) {
+                                            const uint8_t *buf, uint32_t pos, uint64_t u0,
+                                            uint32_t known = kNoSlot) {
     const uint64_t ua = u0 + pos;
     if (ua < C.lo || ua >= C.hi) return;
     uint64_t v8;
-    const int gi = gram_lookup(C, buf, pos, &v8);
-    if (gi < 0) return;
+    int gi = (int)known;
+    if (known == kNoSlot) {
+        gi = gram_lookup(C, buf, pos, &v8);
+        if (gi < 0) return;
+    } else {
+        v8 = ld8(buf, pos);
+    }
     const ulonglong2 c = make_ulonglong2(cand_pack(ua - C.mis, (uint32_t)gi, kLenAll), v8);
     const uint32_t s = atomicAdd(w.mcount, 1u);
     if (s < kCandBuf) {
@@ -358,7 +372,7 @@ __device__ __forceinline__ void cand_window(const WinCtx &C, const WarpCtx &w, c
 __device__ __forceinline__ void cand_flush(const WinCtx &C, const WarpCtx &w, const CandList &cc,
                                            const uint8_t *buf, uint64_t u0, uint32_t lane) {
     __syncwarp();
-    const uint32_t cnt = min(*reinterpret_cast<volatile uint32_t *>(w.mcount), kCandBuf);
+    const uint32_t cnt = min(warp_read(w.mcount), kCandBuf);
     if (cnt) {
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(cc.count, (unsigned long long)cnt);
@@ -464,13 +478,13 @@ __device__ __forceinline__ void consume_tile(const WinCtx &C, const WarpCtx &w, 
                 if (DEFER) {
                     cand_window(C, w, *cc, buf, q[qn + lane], u0);
                     __syncwarp();
-                    if (*reinterpret_cast<volatile uint32_t *>(w.mcount) >= kCandBuf - 32)
+                    if (warp_read(w.mcount) >= kCandBuf - 32)
                         cand_flush(C, w, *cc, buf, u0, lane);
                     continue;
                 }
                 process_window<MODE>(C, w, buf, q[qn + lane], u0);
                 __syncwarp();
-                if (*reinterpret_cast<volatile uint32_t *>(w.mcount) >= kMatchCap - 32)
+                if (warp_read(w.mcount) >= kMatchCap - 32)
                     flush(w, lane);
             }
         } else {
@@ -531,18 +545,21 @@ __device__ __forceinline__ void samp_window(const WinCtx &C, const WarpCtx &w, c
     const uint32_t key = *reinterpret_cast<const uint32_t *>(buf + pos);
     const uint32_t smask = (1u << C.smap_bits) - 1u;
     uint32_t idx = (key * kGramMult) >> (32u - C.smap_bits);
-    uint32_t offs = 0;
+    uint32_t offs = 0, known = kNoSlot;
     for (;;) {
         const SampSlot e = C.s2.smap[idx];
         if (e.mask == 0) return;  // a false positive of the bit set
         if (e.key == key) {
             offs = e.mask;
+            known = e.gi;
             break;
         }
         idx = (idx + 1) & smask;
     }
-    for (uint32_t j = 0; j < 4; ++j)
-        if (((offs >> j) & 1u) && pos >= j && pos - j < tile) cand_window(C, w, cc, buf, pos - j, u0);
+    for (uint32_t m = offs; m; m &= m - 1) {
+        const uint32_t j = __ffs(m) - 1u;
+        if (pos >= j && pos - j < tile) cand_window(C, w, cc, buf, pos - j, u0, known);
+    }
 }
 
 // One consumer warp's share of a staged tile in a sampled, deferred scan:
@@ -600,7 +617,7 @@ __device__ __forceinline__ void consume_tile_s4(const WinCtx &C, const WarpCtx &
                 qn -= 32;
                 samp_window(C, w, cc, buf, q[qn + lane], u0, tile);
                 __syncwarp();
-                if (*reinterpret_cast<volatile uint32_t *>(w.mcount) >= kCandBuf - 32)
+                if (warp_read(w.mcount) >= kCandBuf - 32)
                     cand_flush(C, w, cc, buf, u0, lane);
             }
         } else {
@@ -742,7 +759,7 @@ __device__ __forceinline__ void rf_window_g(const WinCtx &C, const WarpCtx &w, c
 __device__ __forceinline__ void rf_cand_flush(const WinCtx &C, const WarpCtx &w,
                                               const CandList &cc, const GText &g, uint32_t lane) {
     __syncwarp();
-    const uint32_t cnt = min(*reinterpret_cast<volatile uint32_t *>(w.mcount), kCandBuf);
+    const uint32_t cnt = min(warp_read(w.mcount), kCandBuf);
     if (cnt) {
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(cc.count, (unsigned long long)cnt);

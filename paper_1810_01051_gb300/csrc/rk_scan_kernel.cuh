@@ -109,7 +109,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
 
     // -------------------------------------- consumer warps
     WinCtx C;
-    C.s2 = make_s2(P.tab, S2S ? ss2 : P.tab.s2_base);
+    C.s2 = make_s2<MODE == kFilterNone>(P.tab, S2S ? ss2 : P.tab.s2_base);
     C.lo = P.mis + P.x_begin;
     C.hi = P.mis + P.x_end;
     C.mis = P.mis;
@@ -118,6 +118,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
     C.pid_shift = RK_KEY_OFFSET_BITS;
     C.q = P.tab.q;
     C.gram_bits = P.tab.gram_bits;
+    C.gram_mult = P.tab.gram_mult;
     C.base_log2 = P.tab.base_log2;
     C.n_lengths = P.tab.n_lengths;
     C.smap_bits = P.tab.smap_bits;

@@ -329,21 +329,21 @@ __device__ __forceinline__ bool rf_survivor_warp(const WinCtx &C, const WarpCtx 
         }
         __syncwarp();
         // set-aside positions, a full round of 32 at a time
-        for (uint32_t xn = *reinterpret_cast<volatile uint32_t *>(xb.count); xn >= 32u; xn -= 32u) {
+        for (uint32_t xn = warp_read(xb.count); xn >= 32u; xn -= 32u) {
             rf_position<KIND, DEFER>(C, w, cc, g, xb.pos[xn - 32u + lane]);
             __syncwarp();
             if (lane == 0) *reinterpret_cast<volatile uint32_t *>(xb.count) = xn - 32u;
         }
         __syncwarp();
         // (a buffer that fills up mid-round sends the rest straight out)
-        if (*reinterpret_cast<volatile uint32_t *>(w.mcount) >= (DEFER ? kCandBuf : kMatchCap) / 2) {
+        if (warp_read(w.mcount) >= (DEFER ? kCandBuf : kMatchCap) / 2) {
             if (DEFER) rf_cand_flush(C, w, *cc, g, lane);
             else flush(w, lane);
         }
         if (!__all_sync(kFull, ok)) break;
     }
     // the set-aside positions left
-    const uint32_t xn = *reinterpret_cast<volatile uint32_t *>(xb.count);
+    const uint32_t xn = warp_read(xb.count);
     if (lane < xn) rf_position<KIND, DEFER>(C, w, cc, g, xb.pos[lane]);
     __syncwarp();
     if (DEFER) rf_cand_flush(C, w, *cc, g, lane);
@@ -471,7 +471,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
 
     // -------------------------------------- survivor warps
     WinCtx C;
-    C.s2 = make_s2(P.tab, S2S ? ss2 : P.tab.s2_base);
+    C.s2 = make_s2<false>(P.tab, S2S ? ss2 : P.tab.s2_base);
     C.lo = lo;
     C.hi = hi;
     C.mis = P.mis;
@@ -480,6 +480,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
     C.pid_shift = RK_KEY_OFFSET_BITS;
     C.q = P.tab.q;
     C.gram_bits = P.tab.gram_bits;
+    C.gram_mult = P.tab.gram_mult;
     C.base_log2 = P.tab.base_log2;
     C.n_lengths = P.tab.n_lengths;
     C.smap_bits = 0;

@@ -4,9 +4,9 @@
 // kernel.  For a pattern set the host builds, in one device allocation:
 //   - stage-1 bit set over the q-byte prefixes of all patterns (q = min(4,
 //     shortest length)), keyed by the prefix read as a little-endian word;
-//   - prefix map: exact q-byte prefix -> distinct lengths of the patterns
-//     that start with it, plus a 32-bit fingerprint set of their next four
-//     bytes;
+//   - prefix map: exact q-byte prefix -> a run per distinct length of the
+//     patterns that start with it (a single pattern is named in its run),
+//     plus a 32-bit fingerprint set of their next four bytes;
 //   - one open-addressing table per pattern length L, keyed by the Rabin
 //     hash h_B(P) = sum_i P[i] * B^(L-1-i) mod (2^61 - 1), B = 2^base_log2,
 //     each slot naming the ids of the patterns of that length and hash;
@@ -281,39 +281,69 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     std::sort(lengths.begin(), lengths.end());
     lengths.erase(std::unique(lengths.begin(), lengths.end()), lengths.end());
 
-    // ---- prefix map: q-byte prefix -> distinct lengths ----------------------
-    std::unordered_map<uint32_t, std::vector<uint32_t>> gram_to_lens;
+    // ---- prefix map: q-byte prefix -> a run per distinct length ------------
+    std::unordered_map<uint32_t, std::vector<std::pair<uint32_t, uint32_t>>> gram_to_lens;
     std::unordered_map<uint32_t, uint32_t> gram_ext;
     gram_to_lens.reserve(k * 2 + 1);
     for (uint32_t i = 0; i < k; ++i) {
         const uint8_t *p = patterns + src_off[i];
         uint32_t key = prefix_key(p, q);
-        gram_to_lens[key].push_back(plen[i]);
+        gram_to_lens[key].emplace_back(plen[i], i);
         uint32_t &ext = gram_ext[key];
         if (plen[i] >= q + 4) ext |= 1u << ext_bit(prefix_key(p + q, 4));
     }
     std::vector<uint32_t> gram_keys;
     gram_keys.reserve(gram_to_lens.size());
     for (auto &kv : gram_to_lens) {
-        auto &v = kv.second;
-        std::sort(v.begin(), v.end());
-        v.erase(std::unique(v.begin(), v.end()), v.end());
+        std::sort(kv.second.begin(), kv.second.end());
         gram_keys.push_back(kv.first);
     }
     std::sort(gram_keys.begin(), gram_keys.end());  // deterministic layout
     uint32_t D = (uint32_t)gram_keys.size();
-    uint32_t gram_bits = std::max<uint32_t>(4, ceil_log2(2ull * D));
+    // A warp's lookup takes as many probes as its unluckiest lane, so the map
+    // is sparse: one slot in eight used (up to 16 KiB), else one in four (one
+    // in two above 2^19 prefixes: a listed candidate holds a slot in 22 bits),
+    // and the multiplier is the one of a few with the fewest probes.
+    const uint64_t sparse = D <= 128 ? 8 : D <= (1u << 19) ? 4 : 2;
+    uint32_t gram_bits = std::max<uint32_t>(4, ceil_log2(sparse * D));
     std::vector<GramSlot> grams(1ull << gram_bits, GramSlot{0, 0, 0, 0});
-    std::vector<uint32_t> gram_lens;
+    std::vector<LenRun> gram_runs;
+    const uint32_t mask = (1u << gram_bits) - 1;
+    uint32_t gram_mult = kGramMult, best = UINT32_MAX;
+    std::vector<uint8_t> used;
+    for (uint32_t i = 0, m = kGramMult; i < (D <= 1024 ? 8u : 1u) && best > 1;
+         ++i, m = m * 5 + 2) {
+        used.assign(1ull << gram_bits, 0);
+        uint32_t longest = 0;  // probes of the last key found
+        for (uint32_t key : gram_keys) {
+            uint32_t idx = (key * m) >> (32 - gram_bits), probes = 1;
+            for (; used[idx]; ++probes) idx = (idx + 1) & mask;
+            used[idx] = 1;
+            longest = std::max(longest, probes);
+        }
+        if (longest < best) {
+            best = longest;
+            gram_mult = m;
+        }
+    }
     for (uint32_t key : gram_keys) {
         const auto &v = gram_to_lens[key];
-        uint32_t idx = (key * kGramMult) >> (32 - gram_bits);
-        uint32_t mask = (1u << gram_bits) - 1;
+        uint32_t idx = (key * gram_mult) >> (32 - gram_bits);
         while (grams[idx].count) idx = (idx + 1) & mask;
-        const uint32_t shorts = v.front() < q + 4 ? kGramShort : 0u;  // v ascends
-        grams[idx] = GramSlot{key, (uint32_t)gram_lens.size(), (uint32_t)v.size() | shorts,
-                              gram_ext[key]};
-        gram_lens.insert(gram_lens.end(), v.begin(), v.end());
+        const uint32_t shorts = v.front().first < q + 4 ? kGramShort : 0u;  // v ascends
+        const uint32_t first = (uint32_t)gram_runs.size();
+        uint32_t n_runs = 0;
+        for (size_t i = 0; i < v.size();) {
+            size_t j = i;
+            while (j < v.size() && v[j].first == v[i].first) ++j;
+            const bool one = j == i + 1;
+            const LenRun r{v[i].first, one ? v[i].second : kManyPids,
+                           one ? (uint32_t)(poff[v[i].second] / 8) : 0u, 0};
+            gram_runs.push_back(r);
+            ++n_runs;
+            i = j;
+        }
+        grams[idx] = GramSlot{key, first, n_runs | shorts, gram_ext[key]};
     }
 
     // ---- stage-1 bit set ---------------------------------------------------
@@ -347,22 +377,35 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     std::vector<uint32_t> simg;
     uint32_t smap_bits = 0, smode = 0, sbits = 0, smask_addr = 0;
     if (sampled) {
-        std::unordered_map<uint32_t, uint32_t> offs;
+        struct Gram {
+            uint32_t mask = 0, gi = 0;
+            bool one = true;  // a single offset and prefix so far
+        };
+        std::unordered_map<uint32_t, Gram> offs;
         offs.reserve(k * 8 + 1);
-        for (uint32_t i = 0; i < k; ++i)
-            for (uint32_t j = 0; j < 4; ++j)
-                offs[prefix_key(patterns + src_off[i] + j, 4)] |= 1u << j;
+        for (uint32_t i = 0; i < k; ++i) {
+            const uint32_t prefix = prefix_key(patterns + src_off[i], 4);
+            uint32_t gi = (prefix * gram_mult) >> (32 - gram_bits);
+            while (grams[gi].key != prefix || !grams[gi].count) gi = (gi + 1) & mask;
+            for (uint32_t j = 0; j < 4; ++j) {
+                Gram &g = offs[prefix_key(patterns + src_off[i] + j, 4)];
+                g.one = g.one && (g.mask == 0 || (g.mask == 1u << j && g.gi == gi));
+                g.mask |= 1u << j;
+                g.gi = gi;
+            }
+        }
         std::vector<uint32_t> skeys;
         skeys.reserve(offs.size());
         for (auto &kv : offs) skeys.push_back(kv.first);
         std::sort(skeys.begin(), skeys.end());
         smap_bits = std::max<uint32_t>(4, ceil_log2(2ull * skeys.size()));
-        smap.assign(1ull << smap_bits, SampSlot{0, 0});
+        smap.assign(1ull << smap_bits, SampSlot{0, 0, 0, 0});
         const uint32_t smask = (1u << smap_bits) - 1;
         for (uint32_t key : skeys) {
             uint32_t idx = (key * kGramMult) >> (32 - smap_bits);
             while (smap[idx].mask) idx = (idx + 1) & smask;
-            smap[idx] = SampSlot{key, offs[key]};
+            const Gram &g = offs[key];
+            smap[idx] = SampSlot{key, g.mask, g.one ? g.gi : kNoSlot, 0};
         }
         // the same layout choice as the prefix bit set, for this key set; a
         // flat one tests three bits per gram (stage 1 tests 4x fewer positions)
@@ -410,15 +453,18 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     Blob b;
     size_t o_filter = b.add(fimg.size() * 4 + 16);
     size_t o_grams = b.add(grams.size() * sizeof(GramSlot));
-    size_t o_glens = b.add(gram_lens.size() * 4 + 4);
+    size_t o_runs = b.add(gram_runs.size() * sizeof(LenRun) + sizeof(LenRun));
+    size_t o_pbytes = b.add(packed + 16);
+    size_t o_smap = b.add(smap.size() * sizeof(SampSlot) + 16);
+    // the hash tables of the lengths and what goes with them: with a prefilter
+    // only windows whose prefix and length several patterns share get there,
+    // so these stay in global memory
     size_t o_ghdr = b.add(group_hdr.size() * sizeof(uint2));
     size_t o_slots = b.add(slots.size() * sizeof(GroupSlot) + sizeof(GroupSlot));
     size_t o_gpids = b.add(group_pids.size() * 4 + 4);
-    size_t o_pbytes = b.add(packed + 16);
     size_t o_poff = b.add(k * 8 + 8);
     size_t o_plen = b.add(k * 4 + 4);
     size_t o_lens = b.add(lengths.size() * 4 + 4);
-    size_t o_smap = b.add(smap.size() * sizeof(SampSlot) + 8);
     size_t o_sfilter = b.add(simg.size() * 4 + 16);  // after the survivor tables: not staged with them
     // the side set right after the main one: the scan stages both with one copy
     size_t o_rfilter = b.add((rimg.size() + rside.size()) * 4 + 16);
@@ -426,7 +472,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     uint8_t *hb = b.bytes.data();
     if (!fimg.empty()) memcpy(hb + o_filter, fimg.data(), fimg.size() * 4);
     memcpy(hb + o_grams, grams.data(), grams.size() * sizeof(GramSlot));
-    if (!gram_lens.empty()) memcpy(hb + o_glens, gram_lens.data(), gram_lens.size() * 4);
+    if (!gram_runs.empty()) memcpy(hb + o_runs, gram_runs.data(), gram_runs.size() * sizeof(LenRun));
     memcpy(hb + o_ghdr, group_hdr.data(), group_hdr.size() * sizeof(uint2));
     if (!slots.empty()) memcpy(hb + o_slots, slots.data(), slots.size() * sizeof(GroupSlot));
     if (!group_pids.empty()) memcpy(hb + o_gpids, group_pids.data(), group_pids.size() * 4);
@@ -443,7 +489,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     TableBlob &tb = *out;
     tb.o_filter = o_filter;
     tb.o_grams = o_grams;
-    tb.o_glens = o_glens;
+    tb.o_runs = o_runs;
     tb.o_ghdr = o_ghdr;
     tb.o_slots = o_slots;
     tb.o_gpids = o_gpids;
@@ -475,7 +521,8 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     d.rfilter_bytes = (uint32_t)((rimg.size() + rside.size()) * 4);
     d.rf_side_off = rside.empty() ? 0u : (uint32_t)(rimg.size() * 4);
     d.rf_shift = rstep ? 30 - (rbits - 5) : 0;
-    d.s2_bytes = (uint32_t)(o_sfilter - o_grams);
+    d.s2_bytes = (uint32_t)((mode == kFilterNone ? o_sfilter : o_ghdr) - o_grams);
+    d.gram_mult = gram_mult;
     tb.n_grams = D;
     tb.filter_log2_bits = mode == kFilterNone ? 0 : fbits;
     tb.sfilter_log2_bits = sampled ? sbits : 0;
@@ -489,7 +536,7 @@ void bind_blob(DevTable *d, const TableBlob &b, const uint8_t *dm) {
     *d = b.meta;
     d->filter = (const uint32_t *)(dm + b.o_filter);
     d->grams = (const GramSlot *)(dm + b.o_grams);
-    d->gram_lens = (const uint32_t *)(dm + b.o_glens);
+    d->gram_runs = (const LenRun *)(dm + b.o_runs);
     d->group_hdr = (const uint2 *)(dm + b.o_ghdr);
     d->slots = (const GroupSlot *)(dm + b.o_slots);
     d->group_pids = (const uint32_t *)(dm + b.o_gpids);

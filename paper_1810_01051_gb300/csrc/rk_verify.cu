@@ -51,13 +51,14 @@ __global__ void __launch_bounds__(kVerifyThreads, 8)
     __syncthreads();
     WarpCtx w{mcount + warp, mbuf[warp], P.keys, P.capacity, P.info};
     WinCtx C{};
-    C.s2 = make_s2(P.tab, S2S ? ss2 : P.tab.s2_base);
+    C.s2 = make_s2<false>(P.tab, S2S ? ss2 : P.tab.s2_base);
     C.mis = P.mis;
     C.n = P.n;
     C.key_prefix = 0;
     C.pid_shift = RK_KEY_OFFSET_BITS;
     C.q = P.tab.q;
     C.gram_bits = P.tab.gram_bits;
+    C.gram_mult = P.tab.gram_mult;
     C.base_log2 = P.tab.base_log2;
     C.n_lengths = P.tab.n_lengths;
 
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 8)
             probe_slot(C, w, win, x + P.mis, x, cand_slot(c.x), cand_class(c.x));
         }
         __syncwarp();
-        if (*reinterpret_cast<volatile uint32_t *>(w.mcount) >= kMatchCap - 32) flush(w, lane);
+        if (warp_read(w.mcount) >= kMatchCap - 32) flush(w, lane);
     }
     flush(w, lane);
 }
