@@ -3,7 +3,7 @@
 //
 // Up to 32 tiles of 2048 keys per resident CTA: one cooperative launch that
 // sorts by cells (sort_cells below): the keys' bits that can be non-zero, as
-// one compact number, are cut into about one cell per key by their top bits;
+// one compact number, are cut into a few cells per key by their top bits;
 // the keys are counted and ranked per cell, scattered to their cell, and put
 // in order within it by comparison.  Keys crowded into few cells (more than
 // kCellMax in one) are sorted by the radix passes below instead, in the same
@@ -481,10 +481,20 @@ __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const
     return true;
 }
 
+// Cells per key (at most; a compact key's fields are rounded up to whole bits,
+// so up to three in four cells are empty): eight up to kManyCells keys, where
+// clearing and adding up the counts costs little and a pattern with most of
+// the matches has more cells to itself, two up to kTwoCells, then one, as the
+// counts outgrow L2.  One cell -> this rule: 10 K keys 27 -> 21 us, 31 K of
+// mostly one pattern 54 -> 23 us, 1 M 120 -> 83 us, 2.5 M 153 -> 124 us; two
+// cells at 10 M: 370 -> 394 us.
+constexpr uint64_t kManyCells = 1u << 18, kTwoCells = 1u << 22;
+constexpr uint32_t kKeysPerCta = 512;
+
 enum CellsResult { kCellsDone, kCellsCrowded, kCellsTimeout };
 
-// M keys over G CTAs of a cooperative launch.  cnt: 2^cb + 1 words, rank: M
-// half words, part: G words of workspace; flag and *bar start at zero.
+// M keys over G CTAs of a cooperative launch.  cnt: 2^cb + 1 words (cb >= 11),
+// rank: M half words, part: G words of workspace; flag and *bar start at zero.
 // kCellsCrowded (the same in every CTA): the keys are untouched.
 __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp, uint64_t M,
                                                   const SortShape &shape, uint32_t *cnt,
@@ -618,15 +628,19 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
 // A single tile is sorted by one CTA alone, without barriers.
 // A fixed number of barriers replaces the chain of look-back waits, whose
 // length grows with the tile count.  An odd pass count ends with a copy
-// back from the second buffer.  CTAs beyond the tile count leave at once.
+// back from the second buffer.  CTAs that the list is too short for leave at
+// once.
 __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
     uint64_t *keys, uint64_t *tmp, unsigned long long *info, uint64_t cap, Shifts sh,
-    SortShape shape, uint32_t *cnt, uint32_t pitch, uint32_t *totals, unsigned int *bar,
-    uint32_t *flag) {
+    SortShape shape, uint32_t *cnt, uint64_t cnt_bytes, uint32_t pitch, uint32_t *totals,
+    unsigned int *bar, uint32_t *flag) {
     uint64_t M;
     uint32_t T;
     if (!sort_count(info, cap, &M, &T)) return;
-    const uint32_t G = min(gridDim.x, T);  // CTAs taking part
+    // CTAs taking part: one per kKeysPerCta keys, so that a short list is not
+    // left to a few SMs (64 K keys, with the cells: 34 -> 27 us)
+    const uint32_t G =
+        T == 1 ? 1u : (uint32_t)min((uint64_t)gridDim.x, (M + kKeysPerCta - 1) / kKeysPerCta);
     if (blockIdx.x >= G) return;
     __shared__ uint32_t wcnt[kWarps][256];
     __shared__ uint32_t dbase[256];
@@ -641,9 +655,11 @@ __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
     }
     unsigned int passed = 0;
     {
-        // 2^cb <= M cells (words), then M ranks (half words), then a word per
-        // CTA: at most 12 of the 16 KiB of look-back words that a tile has
-        const uint32_t cb = 31u - __clz((uint32_t)M);
+        // 2^cb cells (words), then M ranks (half words), then a word per CTA, in
+        // the look-back words' space (16 KiB per tile of the capacity)
+        uint32_t cb = 31u - __clz((uint32_t)M);
+        for (uint32_t more = M <= kManyCells ? 3u : M <= kTwoCells ? 1u : 0u; more; --more)
+            if ((8ull << cb) + 2 * M + 4ull * gridDim.x + 64 <= cnt_bytes) ++cb;
         uint16_t *rank = reinterpret_cast<uint16_t *>(cnt + (1u << cb) + 4);
         uint32_t *part = reinterpret_cast<uint32_t *>(rank + (M + 1) / 2 * 2);
         const CellsResult r = sort_cells(keys, tmp, M, shape, cnt, rank, part, cb, flag, bar, G,
@@ -847,12 +863,13 @@ int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
         if (cudaMemsetAsync(counters, 0, L.ghist_off - L.ctrl_off, stream) != cudaSuccess)
             return RK_ECUDA;
         uint32_t *cnt = reinterpret_cast<uint32_t *>(status);
+        uint64_t cnt_bytes = L.total - L.status_off;
         uint32_t pitch = (uint32_t)L.tiles;
         uint32_t *totals = ghist;
         unsigned int *bar = counters + 32;
         uint32_t *flag = counters;
-        void *args[] = {&d_keys, &tmp, &info,   &capacity, &sh,  &shape,
-                        &cnt,    &pitch, &totals, &bar,      &flag};
+        void *args[] = {&d_keys, &tmp,       &info,  &capacity, &sh,  &shape,
+                        &cnt,    &cnt_bytes, &pitch, &totals,   &bar, &flag};
         if (cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(rk_sort_fused_kernel), g,
                                         kThreads, args, 0, stream) != cudaSuccess) {
             cudaGetLastError();

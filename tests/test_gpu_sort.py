@@ -65,3 +65,31 @@ def test_sort_spreads(spread, m, n, k):
             assert not got[keys.size:].any()  # nothing past the list is touched
     finally:
         rk.rk_destroy(table)
+
+
+@pytest.mark.parametrize("spread", ["even", "one_id"])
+@pytest.mark.parametrize("m", [511 * 8, 4096, 4097, (1 << 18) - 1, 1 << 18, (1 << 18) + 1])
+@pytest.mark.parametrize("spare", [0, 1, 400_000])
+def test_sort_cell_counts(spread, m, spare):
+    """Sizes where the number of CTAs and of cells per key change; the cells also
+    depend on the workspace, so on the room beyond the list."""
+    n, k = 1 << 30, 100
+    rng = np.random.default_rng(m + spare)
+    keys = make(spread, m + m // 8, n, k, rng)[:m]
+    table = rk.rk_build([b"%06d" % i for i in range(k)])
+    try:
+        cap = keys.size + spare
+        d = torch.zeros(cap, dtype=torch.int64, device="cuda")
+        d[:keys.size] = torch.from_numpy(keys.view(np.int64)).cuda()
+        info = torch.tensor([keys.size, 0], dtype=torch.int64, device="cuda")
+        wsb = rk.rk_workspace_bytes(table, cap)
+        ws = torch.full((wsb + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+        rk.rk_sort_device(table, n, d, cap, info, ws, wsb)
+        torch.cuda.synchronize()
+        got = d.cpu().numpy().view(np.uint64)
+        assert int(info[1]) == rk.RK_OK
+        assert np.array_equal(got[:keys.size], np.sort(keys))
+        assert not got[keys.size:].any()
+        assert bool((ws[wsb:] == 0xA5).all())  # nothing past the workspace
+    finally:
+        rk.rk_destroy(table)
