@@ -128,6 +128,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
     const uint32_t fmask = P.tab.filter_mask;
     const uint32_t qmask = P.tab.q == 4 ? 0xFFFFFFFFu : (1u << (8u * P.tab.q)) - 1u;
     const uint32_t last = P.tile / 16u - 1u;
+    const GText gt{P.base, P.n16};
 
     for (uint64_t i = 0; i < my_tiles; ++i) {
         const uint32_t s = (uint32_t)(i % P.stages);
@@ -143,13 +144,14 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
         const uint32_t nchunks = (uint32_t)((wend - u0 + 15) / 16);
         if constexpr (SAMP == 1)
             consume_tile_s4<MODE>(C, w, q, buf, u0, nchunks, P.tile, sfilt, fmask, lane4, warp, nw,
-                                  lane, P.cand);
+                                  lane, P.cand, gt);
         else
             consume_tile<MODE, Q4, DEFER>(C, w, q, buf, u0, nchunks, last, sfilt, fmask, lane4,
-                                          qmask, warp, nw, lane, &P.cand);
+                                          qmask, warp, nw, lane, &P.cand, &gt);
         if (lane == 0) mbar_arrive(&empty[s]);
     }
-    if (!DEFER) flush(w, lane);  // (a deferred scan flushes its candidates per tile)
+    if (DEFER) cand_flush(C, w, P.cand, gt, lane);
+    else flush(w, lane);
 }
 
 template <int MODE, bool Q4, int MAXW, bool DEFER, int SAMP>

@@ -337,7 +337,7 @@ __device__ __forceinline__ bool rf_survivor_warp(const WinCtx &C, const WarpCtx 
         __syncwarp();
         // (a buffer that fills up mid-round sends the rest straight out)
         if (warp_read(w.mcount) >= (DEFER ? kCandBuf : kMatchCap) / 2) {
-            if (DEFER) rf_cand_flush(C, w, *cc, g, lane);
+            if (DEFER) cand_flush(C, w, *cc, g, lane);
             else flush(w, lane);
         }
         if (!__all_sync(kFull, ok)) break;
@@ -346,7 +346,7 @@ __device__ __forceinline__ bool rf_survivor_warp(const WinCtx &C, const WarpCtx 
     const uint32_t xn = warp_read(xb.count);
     if (lane < xn) rf_position<KIND, DEFER>(C, w, cc, g, xb.pos[lane]);
     __syncwarp();
-    if (DEFER) rf_cand_flush(C, w, *cc, g, lane);
+    if (DEFER) cand_flush(C, w, *cc, g, lane);
     else flush(w, lane);
     return __all_sync(kFull, ok);
 }
