@@ -250,8 +250,10 @@ int rk_scan_launches(const rk_table *t, uint64_t n, uint64_t workspace_bytes,
  *   d_workspace  16-byte aligned; at least rk_workspace_bytes(t, capacity)
  *                bytes when capacity >= 2 (the sort's).  With
  *                rk_workspace_bytes(t, capacity) + rk_scan_workspace_bytes(t, n)
- *                bytes the scan part runs as rk_scan_device_ws, its list
- *                placed after the sort's workspace.
+ *                bytes the scan part may run as rk_scan_device_ws, its list
+ *                placed after the sort's workspace (short texts, and tables
+ *                whose scan is faster so, complete their survivors in the
+ *                scan).
  * Errors: as rk_scan_device and rk_sort_device.                              */
 int rk_search_device(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t *d_keys,
                      uint64_t capacity, uint64_t *d_info, void *d_workspace,

@@ -157,6 +157,28 @@ int deferred_scan(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t
 
 }  // namespace
 
+namespace {
+
+// Whether a search completes its survivors inside the scan even when it has
+// room for a candidate list.  The second kernel and the list's clear cost about
+// 8 us whatever the text, the scan's own comparisons more per survivor.
+//   - survivor tables in shared memory: prefix filters always (100 words of
+//     3..12, 64 MiB: 150 us in the scan, 180 us with the list, 256 MiB: 562 and
+//     624 us), role filters up to kInScanRoles bytes (100 words of 4..32, 1 MiB:
+//     14 and 22 us, 32 MiB: 36 and 40, 256 MiB: 171 and 165; DNA probes of
+//     25..800, 32 MiB: 86 and 92, 64 MiB: 144 and 129);
+//   - tables in L2: only sampled ones (the scan then tests every position) up
+//     to kInScanSampled (10,000 signatures, 1 MiB: 16 and 23 us, 8 MiB: 32 and
+//     32); role filters lose from 1 MiB on (1000 signatures: 28 and 25 us).
+constexpr uint64_t kInScanRoles = 48ull << 20, kInScanSampled = 4ull << 20;
+
+bool complete_in_scan(const rk_table *t, uint64_t n) {
+    if (t->tune.s2_smem && t->dev.sample != 4) return !t->dev.rf_step || n <= kInScanRoles;
+    return t->dev.sample == 4 && n <= kInScanSampled;
+}
+
+}  // namespace
+
 extern "C" int rk_scan_launches(const rk_table *t, uint64_t n, uint64_t workspace_bytes,
                                 uint32_t *launches) {
     if (!t || !launches) return RK_EINVAL;
@@ -242,7 +264,7 @@ extern "C" int rk_search_device(const rk_table *t, const uint8_t *d_text, uint64
     // the survivors' verification to a second kernel
     const uint64_t sort_bytes = capacity >= 2 ? sort_workspace_bytes(capacity) : 0;
     CandList cl;
-    if (d_workspace && workspace_bytes > sort_bytes &&
+    if (d_workspace && workspace_bytes > sort_bytes && !complete_in_scan(t, n) &&
         cand_list(t, n, reinterpret_cast<uint8_t *>(d_workspace) + sort_bytes,
                   workspace_bytes - sort_bytes, &cl))
         rc = deferred_scan(t, d_text, n, d_keys, capacity, d_info, cl,
@@ -282,8 +304,9 @@ extern "C" int rk_search(const rk_table *tc, const uint8_t *h_text, uint64_t n, 
     const uint64_t scan_bytes = can_defer(t) ? scan_ws_layout(n).total : 0;
     if ((rc = ensure(&t->h_ws, &t->h_ws_cap, sort_bytes + scan_bytes))) return rc;
     CandList cl;
-    const bool defer = scan_bytes && cand_list(t, n, reinterpret_cast<uint8_t *>(t->h_ws) + sort_bytes,
-                                               scan_bytes, &cl);
+    const bool defer = scan_bytes && !complete_in_scan(t, n) &&
+                       cand_list(t, n, reinterpret_cast<uint8_t *>(t->h_ws) + sort_bytes,
+                                 scan_bytes, &cl);
 
     // Copy the text in chunks on one stream while the other scans the windows
     // whose bytes (window + longest pattern - 1) have arrived.
