@@ -13,8 +13,49 @@ namespace rk {
 namespace {
 
 constexpr uint32_t kVerifyThreads = 256;
+constexpr uint32_t kVerifyBlocks = 5;  // per SM
 constexpr uint32_t kVerifyWarps = kVerifyThreads / 32;
 constexpr uint32_t kVerifySmemMax = 32u << 10;  // survivor tables staged in shared memory
+
+// A window from the list: compared 32 bytes at a time, the text's loads and the
+// pattern's issued together, so that a pattern of up to 40 bytes costs one
+// round trip.  Here the loads' latency is what there is to save (10 M
+// candidates of 8..64 bytes: 616 -> 446 us); in the scans, whose few survivor
+// warps are short of issue slots, the extra instructions cost more (1 GiB of
+// words 1393 -> 1441 us).
+struct LText : WText {};
+
+__device__ __forceinline__ bool verify(const LText &w, uint64_t pos, const uint8_t *pat,
+                                       uint32_t L) {
+    const uint64_t *pw = reinterpret_cast<const uint64_t *>(pat);
+    const uint64_t last = (pos + L - 1) >> 2;  // the last word that holds a window byte
+    const uint32_t s = (uint32_t)(pos & 3u) * 8u;
+    uint64_t d = w.first8 ^ pw[0];
+    if (L < 8) d &= (1ull << (8u * L)) - 1ull;
+    for (uint32_t i = 8; i < L; i += 32) {
+        const uint64_t a = (pos + i) >> 2;
+        const uint32_t *tw = reinterpret_cast<const uint32_t *>(w.g.base) + a;
+        const uint32_t lim = (uint32_t)(last - a);
+        uint32_t t[9];
+        uint64_t p[4];
+#pragma unroll
+        for (uint32_t j = 0; j < 9; ++j) t[j] = __ldg(tw + min(j, lim));
+#pragma unroll
+        for (uint32_t b = 0; b < 4; ++b) p[b] = i + 8u * b < L ? pw[i / 8u + b] : 0;
+#pragma unroll
+        for (uint32_t b = 0; b < 4; ++b) {
+            const uint32_t o = i + 8u * b;
+            if (o >= L) continue;
+            const uint32_t lo = __funnelshift_r(t[2 * b], t[2 * b + 1], s),
+                           hi = __funnelshift_r(t[2 * b + 1], t[2 * b + 2], s);
+            uint64_t x = (((uint64_t)hi << 32) | lo) ^ p[b];
+            if (L - o < 8) x &= (1ull << (8u * (L - o))) - 1ull;
+            d |= x;
+        }
+        if (d) return false;
+    }
+    return d == 0;
+}
 
 struct VerifyParams {
     DevTable tab;
@@ -31,11 +72,12 @@ struct VerifyParams {
 
 // S2S: the survivor tables (P.tab.s2_bytes) are first copied to the block's
 // dynamic shared memory, so each candidate's chain of table loads stays on
-// chip; otherwise they are read through L1/L2.  Eight blocks per SM (32
-// registers a thread): the kernel waits on global loads, and more resident
-// warps hide more of that latency.
+// chip; otherwise they are read through L1/L2.  Five blocks per SM: the kernel
+// waits on chains of global loads (candidate, slot, run, pattern and text), and
+// the registers that keep a comparison's loads in flight together are worth
+// more than the warps (10 M candidates: six blocks 502 us, five 446 us).
 template <bool S2S>
-__global__ void __launch_bounds__(kVerifyThreads, 8)
+__global__ void __launch_bounds__(kVerifyThreads, kVerifyBlocks)
     rk_verify_kernel(const __grid_constant__ VerifyParams P) {
     extern __shared__ __align__(128) uint8_t ss2[];
     __shared__ uint32_t mcount[kVerifyWarps];
@@ -70,7 +112,7 @@ __global__ void __launch_bounds__(kVerifyThreads, 8)
         if (i < nc) {
             const ulonglong2 c = P.list[i];
             const uint64_t x = cand_x(c.x);
-            const WText win{P.text, x + P.mis, c.y};
+            const LText win{{P.text, x + P.mis, c.y}};
             probe_slot(C, w, win, x + P.mis, x, cand_slot(c.x), cand_class(c.x));
         }
         __syncwarp();
@@ -97,7 +139,7 @@ int launch_verify(const rk_table *t, const uint8_t *d_text, uint64_t n, const Ca
     p.keys = d_keys;
     p.capacity = capacity;
     p.info = reinterpret_cast<unsigned long long *>(d_info);
-    const uint32_t grid = (uint32_t)t->sm_count * 8;
+    const uint32_t grid = (uint32_t)t->sm_count * kVerifyBlocks;
     // tables up to 32 KiB go to shared memory (with the static 8 KiB, at
     // least five blocks of 256 threads per SM); larger ones stay in L2
     const uint32_t s2 = t->dev.s2_bytes;
