@@ -24,7 +24,7 @@ int scan_args_ok(const rk_table *t, const uint8_t *d_text, uint64_t n, const uin
 }
 
 // ---- A2 on its own: Rabin hash of every window from prefix hashes ----------
-// A CTA takes a tile of kHashTile bytes.  With P[i] the hash of the tile's
+// A CTA of T threads takes a tile of 16 T bytes.  With P[i] the hash of the tile's
 // first i bytes, the window of L bytes at i has the hash P[i + L] - P[i] * B^L,
 // and every product by a power of B = 2^k is a 61-bit rotation.  Each thread
 // hashes 16 bytes, the threads' hashes are scanned (shuffles, then the warps'
@@ -33,31 +33,29 @@ int scan_args_ok(const rk_table *t, const uint8_t *d_text, uint64_t n, const uin
 // windows are then written in order, a warp's 32 hashes side by side.
 //
 // One byte read and eight written per window; bound by the integer pipes (two
-// rotations and two reductions mod p per byte) and the writes.  128 MiB of text,
-// 16-byte windows: 332 us, 3.6 TB/s (a rolling update per thread over 64
-// windows of its own, whose writes lie 512 bytes from its neighbour's: 1553 us).
-constexpr uint32_t kHashThreads = 512;
-constexpr uint32_t kHashTile = 16 * kHashThreads;  // bytes
-constexpr uint32_t kHashWarps = kHashThreads / 32;
-
+// rotations and two reductions mod p per byte: 90 % busy), the writes take half
+// the time.  128 MiB of text, 16-byte windows: 302 us, 4.0 TB/s, with tiles of
+// 128 threads (256: 310 us, 512: 332 us: every thread adds up the warps before
+// its own).  A rolling update per thread over 64 windows of its own, whose
+// writes lie 512 bytes from its neighbour's: 1553 us.
 __host__ __device__ constexpr uint32_t hash_slot(uint32_t i) { return i + (i >> 4); }
-constexpr uint32_t kHashSmem = 8 * (hash_slot(kHashTile) + 1);
+constexpr uint32_t hash_smem(uint32_t threads) { return 8 * (hash_slot(16 * threads) + 1); }
 
 // Windows per tile for windows of L bytes: whole warps.
-__host__ __device__ constexpr uint32_t hash_windows(uint32_t L) {
-    return (kHashTile - L + 1) / 32 * 32;
+__host__ __device__ constexpr uint32_t hash_windows(uint32_t threads, uint32_t L) {
+    return (16 * threads - L + 1) / 32 * 32;
 }
 
 // K8: B = 2^8 (the default base).
-template <bool K8>
-__global__ void __launch_bounds__(kHashThreads, 3)
+template <bool K8, uint32_t T>
+__global__ void __launch_bounds__(T, 1536 / T)
     rk_window_hash_kernel(GText text, uint64_t mis, uint64_t nw, uint32_t L, uint32_t base_log2,
                           uint64_t *out) {
     extern __shared__ __align__(16) uint64_t prefix[];
-    __shared__ uint64_t wtot[kHashWarps];
+    __shared__ uint64_t wtot[T / 32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t k = K8 ? 8u : base_log2;
-    const uint32_t W = hash_windows(L);
+    const uint32_t W = hash_windows(T, L);
     const uint64_t x0 = blockIdx.x * (uint64_t)W;
 
     // this thread's 16 bytes (past the text: any bytes, used by no window)
@@ -94,11 +92,11 @@ __global__ void __launch_bounds__(kHashThreads, 3)
         h = rotl61(h, k) + (((j < 8 ? b0 : b1) >> (8 * (j & 7))) & 0xFFu);
         if (h >= kP61) h -= kP61;
     }
-    if (tid == kHashThreads - 1) prefix[hash_slot(kHashTile)] = h;
+    if (tid == T - 1) prefix[hash_slot(16 * T)] = h;
     __syncthreads();
     const uint32_t sL = (uint32_t)((uint64_t)k * L % 61);
     const uint32_t count = (uint32_t)min((uint64_t)W, nw - x0);
-    for (uint32_t i = tid; i < count; i += kHashThreads)
+    for (uint32_t i = tid; i < count; i += T)
         out[x0 + i] = submod61(prefix[hash_slot(i + L)], rotl61(prefix[hash_slot(i)], sL));
 }
 
@@ -361,6 +359,28 @@ extern "C" int rk_search(const rk_table *tc, const uint8_t *h_text, uint64_t n, 
     return RK_OK;
 }
 
+namespace {
+
+// Windows of up to kShortHash bytes take small tiles (an eighth of one at most
+// is then hashed twice).
+constexpr uint32_t kShortHash = 256;
+
+template <uint32_t T>
+int launch_hashes(const GText &text, uint64_t mis, uint64_t nw, uint32_t L, uint32_t base_log2,
+                  uint64_t *d_hashes, cudaStream_t st) {
+    const uint32_t W = hash_windows(T, L);
+    const auto fn = base_log2 == 8 ? rk_window_hash_kernel<true, T> : rk_window_hash_kernel<false, T>;
+    if (hash_smem(T) > (48u << 10) &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)hash_smem(T)) != cudaSuccess)
+        return RK_ECUDA;
+    fn<<<(uint32_t)((nw + W - 1) / W), T, hash_smem(T), st>>>(text, mis, nw, L, base_log2,
+                                                              d_hashes);
+    return cudaGetLastError() == cudaSuccess ? RK_OK : RK_ECUDA;
+}
+
+}  // namespace
+
 extern "C" int rk_window_hashes_device(const uint8_t *d_text, uint64_t n, uint32_t L,
                                        uint32_t base_log2, uint64_t *d_hashes, void *stream) {
     if (L < 1 || L > RK_MAX_PATTERN_LEN || base_log2 < 1 || base_log2 > 60) return RK_EINVAL;
@@ -372,15 +392,9 @@ extern "C" int rk_window_hashes_device(const uint8_t *d_text, uint64_t n, uint32
     const GText text{reinterpret_cast<const uint8_t *>(addr & ~uintptr_t(15)),
                      (mis + n + 15) & ~uint64_t(15)};
     const uint64_t nw = n - L + 1;
-    const uint32_t W = hash_windows(L);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const auto fn = base_log2 == 8 ? rk_window_hash_kernel<true> : rk_window_hash_kernel<false>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHashSmem) !=
-        cudaSuccess)
-        return RK_ECUDA;
-    fn<<<(uint32_t)((nw + W - 1) / W), kHashThreads, kHashSmem, st>>>(text, mis, nw, L, base_log2,
-                                                                      d_hashes);
-    return cudaGetLastError() == cudaSuccess ? RK_OK : RK_ECUDA;
+    if (L <= kShortHash) return launch_hashes<128>(text, mis, nw, L, base_log2, d_hashes, st);
+    return launch_hashes<512>(text, mis, nw, L, base_log2, d_hashes, st);
 }
 
 extern "C" int rk_debug_scan_withheld(const rk_table *t, const uint8_t *d_text, uint64_t n,
