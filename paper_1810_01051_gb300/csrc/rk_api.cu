@@ -143,11 +143,11 @@ bool cand_list(const rk_table *t, uint64_t n, void *ws, uint64_t ws_bytes, CandL
 // `mid` (optional) is recorded between the two launches.
 int deferred_scan(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t *d_keys,
                   uint64_t capacity, uint64_t *d_info, const CandList &cl, cudaStream_t st,
-                  cudaEvent_t mid = nullptr) {
+                  cudaEvent_t mid = nullptr, ZeroWords zero = {}) {
     if (cudaMemsetAsync(d_info, 0, 2 * sizeof(uint64_t), st) != cudaSuccess ||
         cudaMemsetAsync(cl.count, 0, sizeof(unsigned long long), st) != cudaSuccess)
         return RK_ECUDA;
-    int rc = launch_scan(t, d_text, n, 0, n, d_keys, capacity, d_info, st, &cl);
+    int rc = launch_scan(t, d_text, n, 0, n, d_keys, capacity, d_info, st, &cl, zero);
     if (rc) return rc;
     if (mid && cudaEventRecord(mid, st) != cudaSuccess) return RK_ECUDA;
     return launch_verify(t, d_text, n, cl, d_keys, capacity, d_info, st);
@@ -261,17 +261,20 @@ extern "C" int rk_search_device(const rk_table *t, const uint8_t *d_text, uint64
     // a workspace that also holds a scan workspace after the sort's defers
     // the survivors' verification to a second kernel
     const uint64_t sort_bytes = capacity >= 2 ? sort_workspace_bytes(capacity) : 0;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const ZeroWords zero = sort_control(t, n, capacity, d_workspace);
     CandList cl;
     if (d_workspace && workspace_bytes > sort_bytes && !complete_in_scan(t, n) &&
         cand_list(t, n, reinterpret_cast<uint8_t *>(d_workspace) + sort_bytes,
                   workspace_bytes - sort_bytes, &cl))
-        rc = deferred_scan(t, d_text, n, d_keys, capacity, d_info, cl,
-                           reinterpret_cast<cudaStream_t>(stream));
+        rc = deferred_scan(t, d_text, n, d_keys, capacity, d_info, cl, st, nullptr, zero);
+    else if (cudaMemsetAsync(d_info, 0, 2 * sizeof(uint64_t), st) != cudaSuccess)
+        rc = RK_ECUDA;
     else
-        rc = rk_scan_device(t, d_text, n, d_keys, capacity, d_info, stream);
+        rc = launch_scan(t, d_text, n, 0, n, d_keys, capacity, d_info, st, nullptr, zero);
     if (rc) return rc;
-    return launch_sort(t, n, d_keys, capacity, d_info, d_workspace, workspace_bytes,
-                       reinterpret_cast<cudaStream_t>(stream));
+    return launch_sort(t, n, d_keys, capacity, d_info, d_workspace, workspace_bytes, st,
+                       zero.n != 0);
 }
 
 extern "C" int rk_search(const rk_table *tc, const uint8_t *h_text, uint64_t n, uint64_t *h_keys,

@@ -34,6 +34,7 @@ struct BatchDesc {
     uint32_t work_counter;
     uint32_t pad;
 };
+static_assert(sizeof(BatchDesc) == 16, "the result header follows, cleared with the counter");
 
 struct BatchParams {
     const BatchItem *items;
@@ -46,6 +47,7 @@ struct BatchParams {
     uint32_t fslot;      // bytes reserved per stage for a bit set
     uint32_t s2slot;     // bytes reserved per stage for survivor tables (0: read from L2)
     uint32_t ob, pb;     // offset and id field widths of a key
+    ZeroWords zero;      // the sort's control words, cleared by the first CTA
 };
 
 struct BatchLayout {
@@ -104,6 +106,8 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
         fence_mbar_init();
     }
     if (tid < nw) mcount[tid] = 0;
+    if (blockIdx.x == 0)
+        for (uint32_t i = tid; i < P.zero.n; i += blockDim.x) P.zero.p[i] = 0;
     __syncthreads();
 
     if (warp == nw) {  // ---------------- producer warp
@@ -504,16 +508,17 @@ int upload(rk_batch *b, cudaStream_t st) {
 
 // Enqueue one full batch run (scan, sort, offsets) on st.
 int enqueue(rk_batch *b, cudaStream_t st, bool scan_only) {
-    const BatchParams p = params_of(b);
+    BatchParams p = params_of(b);
+    p.zero = sort_control(b->sm_count, b->opts.capacity, b->d_ws);
     const uint32_t grid = (uint32_t)b->sm_count * b->opts.ctas_per_sm;
-    if (cudaMemsetAsync(b->d_info, 0, 16, st) != cudaSuccess) return RK_ECUDA;
-    if (cudaMemsetAsync(&b->d_desc->work_counter, 0, 4, st) != cudaSuccess) return RK_ECUDA;
+    // the chunk counter and, right after the description, the result header
+    if (cudaMemsetAsync(&b->d_desc->work_counter, 0, 8 + 16, st) != cudaSuccess) return RK_ECUDA;
     if (dispatch(b->ts->filter_mode, b->ts->all_q4, false, p, grid, b->smem, st) != cudaSuccess)
         return RK_ECUDA;
     if (scan_only) return RK_OK;
     const SortShape shape{b->ob + b->pb + b->tb, 0, 0};
     int rc = launch_sort_shape(b->sm_count, shape, b->d_keys, b->opts.capacity, b->d_info, b->d_ws,
-                               b->ws_bytes, st);
+                               b->ws_bytes, st, p.zero.n != 0);
     if (rc) return rc;
     const uint32_t blocks = std::max<uint32_t>(1, (b->opts.max_items + 1 + 255) / 256);
     rk_batch_offsets_kernel<<<std::min<uint32_t>(blocks, 1024), 256, 0, st>>>(
@@ -601,7 +606,7 @@ extern "C" int rk_batch_create(const rk_tableset *ts, const rk_batch_opts *opts,
     const uint64_t o_items = 0;
     const uint64_t o_chunks = ws_align(o_items + sizeof(BatchItem) * o.max_items);
     const uint64_t o_desc = ws_align(o_chunks + sizeof(uint4) * b->max_chunks);
-    const uint64_t o_info = ws_align(o_desc + sizeof(BatchDesc));
+    const uint64_t o_info = o_desc + sizeof(BatchDesc);
     const uint64_t o_off = ws_align(o_info + 16);
     const uint64_t o_keys = ws_align(o_off + 8ull * (o.max_items + 1));
     const uint64_t o_ws = ws_align(o_keys + 8ull * cap);

@@ -230,11 +230,19 @@ struct CandList {
     unsigned long long *count;  // candidates offered (zeroed before the scan; may exceed cap)
 };
 
+// Words of device memory that a kernel clears at its start for the next one in
+// the stream (a separate clear costs about 2 us, much of a short search).
+struct ZeroWords {
+    uint32_t *p;
+    uint32_t n;
+};
+
 // Scan windows whose start x lies in [x_begin, x_end) of a text of n bytes
 // (bytes up to min(n, x_end + lmax - 1) must be resident); adds to d_info.
+// Clears `zero`, unless there is nothing to scan.
 int launch_scan(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t x_begin,
                 uint64_t x_end, uint64_t *d_keys, uint64_t capacity, uint64_t *d_info,
-                cudaStream_t stream, const CandList *cand = nullptr);
+                cudaStream_t stream, const CandList *cand = nullptr, ZeroWords zero = {});
 
 // launch_scan with an explicit wait limit; `withhold` makes the producer
 // issue no copy (diagnostics: every consumer wait then runs out).  With a
@@ -243,7 +251,7 @@ int launch_scan(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t x
 int launch_scan_opts(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t x_begin,
                      uint64_t x_end, uint64_t *d_keys, uint64_t capacity, uint64_t *d_info,
                      cudaStream_t stream, uint64_t timeout_ns, bool withhold,
-                     const CandList *cand = nullptr);
+                     const CandList *cand = nullptr, ZeroWords zero = {});
 
 // Tables whose survivors can be verified in a second pass: a stage-1 filter
 // and prefix-map slot indices below 2^24.
@@ -254,8 +262,15 @@ bool can_defer(const rk_table *t);
 int launch_verify(const rk_table *t, const uint8_t *d_text, uint64_t n, const CandList &cand,
                   uint64_t *d_keys, uint64_t capacity, uint64_t *d_info, cudaStream_t stream);
 
+// The control words of the sort that these arguments lead to, for a scan
+// before it to clear (n 0: none, or nothing to sort).
+ZeroWords sort_control(const rk_table *t, uint64_t n, uint64_t capacity, void *d_ws);
+ZeroWords sort_control(int sm_count, uint64_t capacity, void *d_ws);
+
+// `cleared`: the words of sort_control are zero already.
 int launch_sort(const rk_table *t, uint64_t n, uint64_t *d_keys, uint64_t capacity,
-                const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream);
+                const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream,
+                bool cleared = false);
 
 // The bits of a sort's keys that can be non-zero: lo_bits from bit 0 on and,
 // above them, hi_bits from bit hi_shift on.
@@ -267,7 +282,8 @@ struct SortShape {
 // to 32 tiles per resident CTA in one cooperative launch, larger ones by one
 // look-back kernel per 8-bit digit.
 int launch_sort_shape(int sm_count, const SortShape &shape, uint64_t *d_keys, uint64_t capacity,
-                      const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream);
+                      const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream,
+                      bool cleared = false);
 
 uint64_t sort_workspace_bytes(uint64_t capacity);
 

@@ -50,9 +50,9 @@ constexpr uint64_t kWaitTimeoutNs = 4000000000ull;  // 4 s per wait (default)
 
 int launch_scan(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t x_begin,
                 uint64_t x_end, uint64_t *d_keys, uint64_t capacity, uint64_t *d_info,
-                cudaStream_t stream, const CandList *cand) {
+                cudaStream_t stream, const CandList *cand, ZeroWords zero) {
     return launch_scan_opts(t, d_text, n, x_begin, x_end, d_keys, capacity, d_info, stream,
-                            kWaitTimeoutNs, false, cand);
+                            kWaitTimeoutNs, false, cand, zero);
 }
 
 cudaError_t allow_smem(const void *fn, std::atomic<uint64_t> *done) {
@@ -76,7 +76,7 @@ bool can_defer(const rk_table *t) {
 int launch_scan_opts(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_t x_begin,
                      uint64_t x_end, uint64_t *d_keys, uint64_t capacity, uint64_t *d_info,
                      cudaStream_t stream, uint64_t timeout_ns, bool withhold,
-                     const CandList *cand) {
+                     const CandList *cand, ZeroWords zero) {
     if (x_end > n) x_end = n;
     if (x_begin >= x_end || t->dev.n_patterns == 0) return RK_OK;
     const Tuning &tu = t->tune;
@@ -115,6 +115,7 @@ int launch_scan_opts(const rk_table *t, const uint8_t *d_text, uint64_t n, uint6
     p.timeout_ns = timeout_ns;
     p.withhold = withhold ? 1u : 0u;
     if (cand && can_defer(t)) p.cand = *cand;
+    p.zero = zero;
     uint32_t grid = (uint32_t)(p.n_tiles < max_ctas ? p.n_tiles : max_ctas);
     uint32_t threads = (tu.warps + 1) * 32;
     bool q4 = t->dev.q == 4;

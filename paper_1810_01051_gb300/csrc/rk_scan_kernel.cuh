@@ -24,8 +24,14 @@ struct ScanParams {
     uint32_t tile, stages, halo, warps, s2_smem;
     uint32_t sv_warps;       // role-filter kernel: survivor warps
     uint32_t withhold;       // diagnostics: the producer issues no copy at all
+    ZeroWords zero;          // cleared by the first CTA
     CandList cand;           // deferred verification: candidate list (DEFER kernels)
 };
+
+__device__ __forceinline__ void clear_words(const ZeroWords &z) {
+    if (blockIdx.x == 0)
+        for (uint32_t i = threadIdx.x; i < z.n; i += blockDim.x) z.p[i] = 0;
+}
 
 // MAXW: most consumer warps this instance is launched with; the register
 // budget per thread follows from (MAXW + 1) warps per SM.  S2S: the
@@ -56,6 +62,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t nw = P.warps;
 
+    clear_words(P.zero);
     if (MODE != kFilterNone) {
         const uint4 *src = reinterpret_cast<const uint4 *>(P.tab.filter);
         uint4 *dst = reinterpret_cast<uint4 *>(sfilt);

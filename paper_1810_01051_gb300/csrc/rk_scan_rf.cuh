@@ -377,6 +377,7 @@ __global__ void __launch_bounds__((MAXW + 1) * 32, 1)
     uint8_t *stage0 = smem + lay.stage_off;
     const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    clear_words(P.zero);
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(P.tab.filter);
         uint4 *dst = reinterpret_cast<uint4 *>(smem);

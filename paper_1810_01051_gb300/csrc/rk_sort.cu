@@ -842,7 +842,7 @@ uint64_t sort_workspace_bytes(uint64_t capacity) { return sort_ws_bytes(capacity
 
 int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
                       uint64_t capacity, const uint64_t *d_info, void *d_ws, uint64_t ws_bytes,
-                      cudaStream_t stream) {
+                      cudaStream_t stream, bool cleared) {
     SortShape shape = shape_in;
     Shifts sh = shifts_of(shape);
     if (capacity < 2 || sh.n == 0) return RK_OK;
@@ -860,7 +860,8 @@ int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
     if (const uint32_t g = fused_ctas(sm_count, capacity)) {
         // its barrier and flag are the control words; cell counts and ranks,
         // or digit-major counts (256 x tiles), go to the look-back words' space
-        if (cudaMemsetAsync(counters, 0, L.ghist_off - L.ctrl_off, stream) != cudaSuccess)
+        if (!cleared &&
+            cudaMemsetAsync(counters, 0, L.ghist_off - L.ctrl_off, stream) != cudaSuccess)
             return RK_ECUDA;
         uint32_t *cnt = reinterpret_cast<uint32_t *>(status);
         uint64_t cnt_bytes = L.total - L.status_off;
@@ -900,10 +901,23 @@ int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
 }
 
 int launch_sort(const rk_table *t, uint64_t n, uint64_t *d_keys, uint64_t capacity,
-                const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream) {
+                const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream,
+                bool cleared) {
     if (n == 0 || t->dev.n_patterns == 0) return RK_OK;
     return launch_sort_shape(t->sm_count, plain_shape(n, t->dev.n_patterns), d_keys, capacity,
-                             d_info, d_ws, ws_bytes, stream);
+                             d_info, d_ws, ws_bytes, stream, cleared);
+}
+
+ZeroWords sort_control(int sm_count, uint64_t capacity, void *d_ws) {
+    if (capacity < 2 || !d_ws || !fused_ctas(sm_count, capacity)) return {};
+    const SortWsLayout L = sort_ws_layout(capacity);
+    return {reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(d_ws) + L.ctrl_off),
+            (uint32_t)(L.ghist_off - L.ctrl_off) / 4};
+}
+
+ZeroWords sort_control(const rk_table *t, uint64_t n, uint64_t capacity, void *d_ws) {
+    if (n == 0 || t->dev.n_patterns == 0) return {};
+    return sort_control(t->sm_count, capacity, d_ws);
 }
 
 uint32_t sort_launches(const rk_table *t, uint64_t n, uint64_t capacity) {
