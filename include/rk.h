@@ -187,7 +187,7 @@ int rk_scan_device(const rk_table *t, const uint8_t *d_text, uint64_t n, uint64_
  * place, reading the count from d_info on the device.  Does nothing when
  * d_info[0] > capacity.  n must be the text length given to the scan.
  * Outputs of up to 32 tiles of 2048 keys per resident CTA are sorted by one
- * cooperative launch (all digit passes, grid barriers between phases);
+ * cooperative launch (by cells, grid barriers between phases);
  * larger ones by one decoupled look-back kernel per pass.
  *   d_workspace  at least rk_workspace_bytes(t, capacity) bytes, 16-byte aligned.
  * Errors: RK_EINVAL, RK_ECUDA.                                               */
@@ -372,6 +372,8 @@ typedef struct rk_batch_opts {
     uint64_t max_text_len;     /* longest text, >= 1 (sets offset_bits) */
     uint64_t max_total_bytes;  /* most text bytes in one batch */
     uint64_t capacity;         /* match keys per batch, < 2^32 */
+    /* launch shape; with all four 0: three CTAs of 8 warps per SM and 24 KiB tiles
+     * where their shared memory fits, else (and for any given alone) the defaults named */
     uint32_t warps;            /* consumer warps per CTA (default 16) */
     uint32_t tile_bytes;       /* bytes per tile, multiple of 16, <= 65536 (default 32768) */
     uint32_t stages;           /* tiles in flight per CTA (default 2) */
