@@ -19,17 +19,19 @@
 //             4 bytes on) decide which of the windows it stands for survive.
 //             Survivors are queued per warp and processed one per lane: the
 //             prefix map gives the lengths of the patterns with that prefix
-//             and a fingerprint of their next four bytes.
-//  A2 hash    each surviving window gets the Rabin hash mod 2^61 - 1 of its
-//             first L bytes for each such length L.
+//             and a fingerprint of their next four bytes; a prefix and length
+//             that one pattern has alone goes straight to A4.
+//  A2 hash    any other surviving window gets the Rabin hash mod 2^61 - 1 of
+//             its first L bytes for each such length L.
 //  A3 probe   that hash is looked up in the table of its length group.
 //  A4 verify  each pattern of the matching slot is compared byte for byte
 //             (Section 3.1's compare(P, T + x, m) after hx == hy).
 //  A5 emit    matches collect in a per-warp shared buffer and are appended
 //             to the output with one atomic per warp flush.
 //
-// The survivor-stage tables (prefix map, length groups, pattern bytes) are
-// copied to shared memory when they fit, else read through L1/L2.
+// The survivor-stage tables (prefix map, runs, pattern bytes; without a
+// prefilter the length groups too) are copied to shared memory when they fit,
+// else read through L1/L2.
 //
 // All waits are bounded; on a timeout the kernel records RK_ETIMEOUT in
 // d_info[1], stops issuing copies, waits (bounded) for its copies in flight

@@ -1,9 +1,10 @@
-// Second pass of a deferred scan: A2 hash, A3 probe, A4 verify and A5 emit
+// Second pass of a deferred scan: A4 verify (A2 hash and A3 probe before it
+// where patterns share prefix and length) and A5 emit
 // for every candidate the tiled scan listed (a window whose exact q-byte
 // prefix starts some pattern and whose next four bytes pass that prefix's
 // fingerprint set).  The scan kernel handles one tile at a time, so its
 // survivor rounds hold only the few candidates of one warp's share of a
-// tile and a warp pays for the longest hash among them; here every warp
+// tile and a warp pays for the longest window among them; here every warp
 // takes 32 listed candidates at a time; a window's first 8 bytes come with
 // the candidate, longer windows read the rest from the text in global memory.
 #include "rk_scan_body.cuh"
