@@ -42,7 +42,7 @@ class Matcher:
         scan_b = rk.rk_scan_workspace_bytes(self.table, n)
         while True:
             keys = torch.empty(max(cap, 1), dtype=torch.int64, device=text.device)
-            info = torch.zeros(2, dtype=torch.int64, device=text.device)
+            info = torch.empty(2, dtype=torch.int64, device=text.device)  # the search clears it
             wsb = rk.rk_workspace_bytes(self.table, cap) + scan_b
             ws = torch.empty(max(wsb, 16), dtype=torch.uint8, device=text.device)
             rk.rk_search_device(self.table, text if n else 0, n, keys, cap, info, ws, wsb, st)
