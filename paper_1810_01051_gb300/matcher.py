@@ -34,7 +34,7 @@ class Matcher:
                stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
         """Sorted match keys (id << 40 | x) of a uint8 CUDA tensor.  The
         workspace holds the sort's scratch and the candidate list, so the
-        scan verifies its survivors in a second kernel when the table allows."""
+        scan may verify its survivors in a second kernel (rk_search_device)."""
         assert text.is_cuda and text.dtype == torch.uint8 and text.is_contiguous()
         n = text.numel()
         cap = capacity if capacity is not None else max(1024, n // 256)
