@@ -387,6 +387,15 @@ constexpr uint32_t kCellMax = 1024;
 constexpr uint32_t kOneCellBits = 12;  // cells of the one-CTA sort
 constexpr uint32_t kOneCellMax = 96;   // and the most keys it compares in one
 
+// The bits of a key that its shape says are zero.  A list with one of them set
+// (keys of another table or a longer text) is sorted by the radix passes, whose
+// digits stay in range whatever the key: its cell would lie past the counts.
+__device__ __forceinline__ uint64_t outside_shape(const SortShape &s) {
+    const uint64_t lo = s.lo_bits >= 64 ? ~0ull : (1ull << s.lo_bits) - 1ull;
+    return ~(s.hi_bits ? lo | (((1ull << s.hi_bits) - 1ull) << s.hi_shift) : lo);
+}
+
+// (of a key without such bits)
 __device__ __forceinline__ uint64_t compact_key(uint64_t k, const SortShape &s) {
     const uint64_t lo = s.lo_bits >= 64 ? k : k & ((1ull << s.lo_bits) - 1ull);
     return s.hi_bits ? ((k >> s.hi_shift) << s.lo_bits) | lo : lo;
@@ -424,7 +433,8 @@ __device__ __forceinline__ uint32_t cta_excl(uint32_t v, uint32_t *wsum, uint32_
 }
 
 // Up to kSortTile keys in one CTA, cells in shared memory.  Returns false,
-// with the keys untouched, when a cell holds too many.
+// with the keys untouched, when a cell holds too many or a key is outside the
+// shape.
 __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const SortShape &shape,
                                                uint64_t *sbuf, uint32_t *cell, uint32_t *wsum) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -432,6 +442,7 @@ __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const
     constexpr uint32_t kKeys = kSortTile / kThreads;
     const uint32_t tb = shape.lo_bits + shape.hi_bits;
     const uint32_t cs = tb > kOneCellBits ? tb - kOneCellBits : 0;
+    const uint64_t outside = outside_shape(shape);
     uint64_t key[kKeys];
     uint32_t cr[kKeys];  // cell << 16 | rank in it
 #pragma unroll
@@ -445,7 +456,9 @@ __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const
     bool crowded = false;
 #pragma unroll
     for (uint32_t r = 0; r < kKeys; ++r)
-        if (r * kThreads + tid < M) {
+        if (r * kThreads + tid < M && (key[r] & outside)) {
+            crowded = true;
+        } else if (r * kThreads + tid < M) {
             const uint32_t c = (uint32_t)(compact_key(key[r], shape) >> cs);
             const uint32_t k = atomicAdd(&cell[c], 1u);
             crowded |= k >= kOneCellMax;
@@ -495,7 +508,8 @@ enum CellsResult { kCellsDone, kCellsCrowded, kCellsTimeout };
 
 // M keys over G CTAs of a cooperative launch.  cnt: 2^cb + 1 words (cb >= 11),
 // rank: M half words, part: G words of workspace; flag and *bar start at zero.
-// kCellsCrowded (the same in every CTA): the keys are untouched.
+// kCellsCrowded (the same in every CTA; a cell holds too many keys, or a key is
+// outside the shape): the keys are untouched.
 __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp, uint64_t M,
                                                   const SortShape &shape, uint32_t *cnt,
                                                   uint16_t *rank, uint32_t *part, uint32_t cb,
@@ -506,6 +520,7 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
     const uint32_t C = 1u << cb;
     const uint32_t tb = shape.lo_bits + shape.hi_bits;
     const uint32_t cs = tb > cb ? tb - cb : 0;
+    const uint64_t outside = outside_shape(shape);
     const uint64_t gid = blockIdx.x * (uint64_t)kThreads + tid, stride = (uint64_t)G * kThreads;
     constexpr uint32_t kU = 8;  // keys in flight per thread
 
@@ -516,8 +531,9 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
     // count, and rank each key in its cell; the first key of every thread
     // alone, so that crowded keys are noticed before they queue up on a cell
     if (gid < M) {
-        const uint32_t c = (uint32_t)(compact_key(__ldcg(keys + gid), shape) >> cs);
-        const uint32_t r = atomicAdd(cnt + c, 1u);
+        const uint64_t k = __ldcg(keys + gid);
+        const uint32_t r =
+            k & outside ? kCellMax : atomicAdd(cnt + (uint32_t)(compact_key(k, shape) >> cs), 1u);
         rank[gid] = (uint16_t)r;
         if (r >= kCellMax) *reinterpret_cast<volatile uint32_t *>(flag) = 1;
     }
@@ -529,9 +545,10 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
         for (uint32_t u = 0; u < kU; ++u) k[u] = i0 + u * stride < M ? __ldcg(keys + i0 + u * stride) : 0;
 #pragma unroll
         for (uint32_t u = 0; u < kU; ++u)
-            r[u] = i0 + u * stride < M
-                       ? atomicAdd(cnt + (uint32_t)(compact_key(k[u], shape) >> cs), 1u)
-                       : 0u;
+            r[u] = i0 + u * stride >= M ? 0u
+                   : k[u] & outside
+                       ? kCellMax
+                       : atomicAdd(cnt + (uint32_t)(compact_key(k[u], shape) >> cs), 1u);
 #pragma unroll
         for (uint32_t u = 0; u < kU; ++u)
             if (i0 + u * stride < M) {

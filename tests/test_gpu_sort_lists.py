@@ -1,0 +1,72 @@
+"""GPU parity of rk_sort_device on key lists that no one search gives: keys
+outside the fields that the text length and the pattern count allow."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from gpu_util import require_gpu  # noqa: E402
+from paper_1810_01051_gb300 import rk  # noqa: E402
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+def sort_keys(keys, n, k, spare=0):
+    """keys sorted by rk_sort_device for a text of n bytes and k patterns; the
+    workspace and what lies after it are checked to be kept apart."""
+    table = rk.rk_build([b"%06d" % i for i in range(k)])
+    try:
+        cap = keys.size + spare
+        d = torch.zeros(cap, dtype=torch.int64, device="cuda")
+        d[:keys.size] = torch.from_numpy(keys.view(np.int64)).cuda()
+        info = torch.tensor([keys.size, 0], dtype=torch.int64, device="cuda")
+        wsb = rk.rk_workspace_bytes(table, cap)
+        ws = torch.full((wsb + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+        rk.rk_sort_device(table, n, d, cap, info, ws, wsb)
+        torch.cuda.synchronize()
+        assert int(info[1]) == rk.RK_OK and int(info[0]) == keys.size
+        assert bool((ws[wsb:] == 0xA5).all())
+        got = d.cpu().numpy().view(np.uint64)
+        assert not got[keys.size:].any()
+        return got[:keys.size]
+    finally:
+        rk.rk_destroy(table)
+
+
+def field_order(keys, n, k):
+    """A stable sort by the bytes that the offsets below n and the ids below k
+    occupy: the order of any key list, ascending where those bytes hold the
+    whole key."""
+    lo = -(-int(n - 1).bit_length() // 8) * 8
+    hi = -(-int(k - 1).bit_length() // 8) * 8
+    mask = np.uint64((((1 << hi) - 1) << 40) | ((1 << lo) - 1))
+    return keys[np.argsort(keys & mask, kind="stable")]
+
+
+@pytest.mark.parametrize("bad", ["id", "id of all ones", "offset", "one key of all ones"])
+@pytest.mark.parametrize("m,n,k", [(2, 100, 3), (700, 1 << 20, 7), (2048, 1 << 20, 1),
+                                   (2049, 1 << 20, 7), (70_001, (1 << 30) - 3, 100),
+                                   (700_001, 1 << 24, 3)])
+def test_keys_outside_the_fields(m, n, k, bad):
+    rng = np.random.default_rng(m + len(bad))
+    ids = rng.integers(0, k, m).astype(np.uint64)
+    xs = rng.integers(0, n, m).astype(np.uint64)
+    some = rng.random(m) < 0.3
+    if bad == "id":
+        ids[some] += np.uint64(k)
+    elif bad == "id of all ones":
+        ids[some] = np.uint64((1 << 24) - 1)
+    elif bad == "offset":
+        xs[some] = rng.integers(0, 1 << 40, int(some.sum())).astype(np.uint64)
+    else:
+        ids[m // 2], xs[m // 2] = np.uint64((1 << 24) - 1), np.uint64((1 << 40) - 1)
+    keys = (ids << np.uint64(40)) | xs
+    for spare in (0, 3000):
+        got = sort_keys(keys, n, k, spare)
+        assert np.array_equal(got, field_order(keys, n, k)), (spare, bad)
