@@ -432,6 +432,23 @@ __device__ __forceinline__ uint32_t cta_excl(uint32_t v, uint32_t *wsum, uint32_
     return before + incl - v;
 }
 
+// The keys before key k, which lies at tmp[own], in its cell [b, e): the smaller
+// ones, and of equal ones those at lower places (counted again, as only a list
+// that its caller made has any; a test of j < own in the one loop: 5 M keys, 78 to
+// a cell, 397 us, this 340, smaller keys alone 303; 1.2 to a cell 196, 196, 192).
+__device__ __forceinline__ uint32_t place_in_cell(const uint64_t *tmp, uint32_t b, uint32_t e,
+                                                  uint32_t own, uint64_t k) {
+    uint32_t less = 0, same = 0;
+    for (uint32_t j = b; j < e; ++j) {
+        const uint64_t v = tmp[j];
+        less += v < k;
+        same += v == k;
+    }
+    if (same > 1)
+        for (uint32_t j = b; j < own; ++j) less += tmp[j] == k;
+    return less;
+}
+
 // Up to kSortTile keys in one CTA, cells in shared memory.  Returns false,
 // with the keys untouched, when a cell holds too many or a key is outside the
 // shape.
@@ -487,9 +504,7 @@ __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const
     for (uint32_t r = 0; r < kKeys; ++r)
         if (r * kThreads + tid < M) {
             const uint32_t b = cell[cr[r] >> 16], e = cell[(cr[r] >> 16) + 1];
-            uint32_t less = 0;
-            for (uint32_t j = b; j < e; ++j) less += sbuf[j] < key[r];
-            keys[b + less] = key[r];
+            keys[b + place_in_cell(sbuf, b, e, b + (cr[r] & 0xFFFFu), key[r])] = key[r];
         }
     return true;
 }
@@ -606,7 +621,8 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
     }
     if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
 
-    // each key's place in its cell: the number of smaller keys there
+    // each key's place in its cell: the number of smaller keys there, and of
+    // equal ones before it
     constexpr uint32_t kV = 4;
     for (uint64_t i0 = gid; i0 < M; i0 += kV * stride) {
         uint64_t k[kV];
@@ -622,9 +638,8 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
 #pragma unroll
         for (uint32_t u = 0; u < kV; ++u)
             if (i0 + u * stride < M) {
-                uint32_t less = 0;
-                for (uint32_t j = b[u]; j < e[u]; ++j) less += tmp[j] < k[u];
-                keys[b[u] + less] = k[u];
+                const uint32_t own = (uint32_t)(i0 + u * stride);
+                keys[b[u] + place_in_cell(tmp, b[u], e[u], own, k[u])] = k[u];
             }
     }
     return kCellsDone;

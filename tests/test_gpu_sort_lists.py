@@ -1,5 +1,6 @@
 """GPU parity of rk_sort_device on key lists that no one search gives: keys
-outside the fields that the text length and the pattern count allow."""
+outside the fields that the text length and the pattern count allow, and keys
+that occur more than once."""
 
 import numpy as np
 import pytest
@@ -70,3 +71,19 @@ def test_keys_outside_the_fields(m, n, k, bad):
     for spare in (0, 3000):
         got = sort_keys(keys, n, k, spare)
         assert np.array_equal(got, field_order(keys, n, k)), (spare, bad)
+
+
+@pytest.mark.parametrize("copies", [2, 3, 40])
+@pytest.mark.parametrize("m", [2, 3, 64, 2047, 2048, 2049, 4097, 70_001, (1 << 18) + 5])
+def test_equal_keys(m, copies):
+    """Every copy of a key stays in the list, the field's largest and smallest
+    keys among them."""
+    n, k = 1 << 26, 8
+    rng = np.random.default_rng(m + copies)
+    own = rng.integers(0, n, -(-m // copies)).astype(np.uint64)
+    own |= rng.integers(0, k, own.size).astype(np.uint64) << np.uint64(40)
+    own[0] = (np.uint64(k - 1) << np.uint64(40)) | np.uint64(n - 1)
+    own[-1] = 0 if own.size > 1 else own[-1]
+    keys = rng.permutation(np.repeat(own, copies)[:m])
+    for spare in (0, 3000):
+        assert np.array_equal(sort_keys(keys, n, k, spare), np.sort(keys)), spare
