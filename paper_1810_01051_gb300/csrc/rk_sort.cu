@@ -5,9 +5,8 @@
 // sorts by cells (sort_cells below): the keys' bits that can be non-zero, as
 // one compact number, are cut into a few cells per key by their top bits;
 // the keys are counted and ranked per cell, scattered to their cell, and put
-// in order within it by comparison.  Keys crowded into few cells (more than
-// kCellMax in one) are sorted by the radix passes below instead, in the same
-// launch.
+// in order within it by comparison.  Keys crowded into few cells (kCrowdedMean)
+// are sorted by the radix passes below instead, in the same launch.
 //
 // Radix passes: least significant digit first over 8-bit digits, only those
 // that can be non-zero: those of the offset field (bits below ceil(log2(n)))
@@ -377,13 +376,20 @@ __device__ __forceinline__ void sort_one_tile(uint64_t *keys, uint64_t M, const 
 // number of digits: five grid barriers in place of three per digit, and each
 // key is read four times and written twice, mostly in L2.
 //
-// kCellMax: the comparisons within a cell cost its size squared; at 1024 keys
-// a cell they cost about what the radix passes do, which take over there.
+// The comparisons within a cell cost its size squared: kCrowdedMean is the mean
+// size (as a key meets it) from which on they cost more than the radix passes,
+// which take over there.  Whole sorts, radix passes / cells: 20 K keys at 100 to a
+// cell 60 / 48 us, at 200 60 / 67; 500 K at 78 72 / 67, at 625 70 / 184; 5 M at 97
+// 390 / 340, at 780 368 / 1560.  It is estimated from samples before the keys are
+// counted (without: 5 M keys at 8000 to a cell 348 -> 520 us, spent on noticing);
+// kCellMax is the most in one cell that the count can meet after that (ranks have
+// 16 bits).
 // Measured against the radix passes in one cooperative launch, as whole
 // searches: 10 M keys (4 GiB of bytes, 10,000 patterns) 4.38 -> 3.82 ms, 0.7 M
 // keys (64 MB of words) 270 -> 235 us, 78,000 keys (33 MB) 103 -> 77 us, 400
 // keys (1 MiB of DNA, one CTA) 37.9 -> 29.6 us.
 constexpr uint32_t kCellMax = 1024;
+constexpr uint32_t kCrowdedMean = 110;
 constexpr uint32_t kOneCellBits = 12;  // cells of the one-CTA sort
 constexpr uint32_t kOneCellMax = 96;   // and the most keys it compares in one
 
@@ -521,16 +527,40 @@ constexpr uint32_t kKeysPerCta = 512;
 
 enum CellsResult { kCellsDone, kCellsCrowded, kCellsTimeout };
 
+// Pairs of keys in one cell among the CTA's samples k, one per thread.  seen:
+// kSeen zero words.
+constexpr uint32_t kSeen = 8 * kThreads;
+static_assert(kSeen == kWarps * 256, "the digit counters' shared memory");
+
+__device__ __forceinline__ uint32_t sample_pairs(uint64_t k, const SortShape &shape, uint32_t cs,
+                                                 uint64_t outside, uint32_t *seen, uint32_t *wsum,
+                                                 uint32_t lane, uint32_t warp) {
+    __syncthreads();  // seen is zero
+    uint32_t before = 0;
+    if (!(k & outside)) {
+        const uint32_t c = (uint32_t)(compact_key(k, shape) >> cs) + 1u;
+        uint32_t s = (c * 0x9E3779B1u) >> 22;  // one of kSeen / 2: four per sample
+        for (;;) {
+            const uint32_t o = atomicCAS(seen + s, 0u, c);
+            if (o == 0 || o == c) break;
+            s = (s + 1) % (kSeen / 2);
+        }
+        before = atomicAdd(seen + kSeen / 2 + s, 1u);
+    }
+    return cta_sum(before, wsum, lane, warp);
+}
+
 // M keys over G CTAs of a cooperative launch.  cnt: 2^cb + 1 words (cb >= 11),
-// rank: M half words, part: G words of workspace; flag and *bar start at zero.
-// kCellsCrowded (the same in every CTA; a cell holds too many keys, or a key is
-// outside the shape): the keys are untouched.
+// rank: M half words, part: G words of workspace, seen: kSeen words of shared
+// memory; flag[0], flag[1] (sampled pairs) and *bar start at zero.
+// kCellsCrowded (the same in every CTA; the cells hold too many keys, or a key
+// is outside the shape): the keys are untouched.
 __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp, uint64_t M,
                                                   const SortShape &shape, uint32_t *cnt,
                                                   uint16_t *rank, uint32_t *part, uint32_t cb,
                                                   uint32_t *flag, unsigned int *bar, uint32_t G,
                                                   unsigned int *passed, unsigned long long *info,
-                                                  uint32_t *wsum, int *s_ok) {
+                                                  uint32_t *seen, uint32_t *wsum, int *s_ok) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t C = 1u << cb;
     const uint32_t tb = shape.lo_bits + shape.hi_bits;
@@ -539,9 +569,20 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
     const uint64_t gid = blockIdx.x * (uint64_t)kThreads + tid, stride = (uint64_t)G * kThreads;
     constexpr uint32_t kU = 8;  // keys in flight per thread
 
+    // a CTA's samples are spread over the whole list: neighbours in it come from
+    // one stretch of text, so a run of them would look crowded
+    const uint64_t sample =
+        __ldcg(keys + ((uint64_t)tid * G + blockIdx.x) * M / ((uint64_t)kThreads * G));
+    for (uint32_t i = tid; i < kSeen; i += kThreads) seen[i] = 0;
     for (uint64_t i = gid; i < C / 4; i += stride)
         __stcg(reinterpret_cast<uint4 *>(cnt) + i, make_uint4(0, 0, 0, 0));
+    const uint32_t pairs = sample_pairs(sample, shape, cs, outside, seen, wsum, lane, warp);
+    if (tid == 0 && pairs) atomicAdd(flag + 1, pairs);
     if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
+    // two keys share a cell with a chance of (mean size - 1) / M
+    if ((uint64_t)__ldcg(flag + 1) * M >
+        (uint64_t)G * (kThreads * (kThreads - 1) / 2) * (kCrowdedMean - 1))
+        return kCellsCrowded;
 
     // count, and rank each key in its cell; the first key of every thread
     // alone, so that crowded keys are noticed before they queue up on a cell
@@ -695,7 +736,7 @@ __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
         uint16_t *rank = reinterpret_cast<uint16_t *>(cnt + (1u << cb) + 4);
         uint32_t *part = reinterpret_cast<uint32_t *>(rank + (M + 1) / 2 * 2);
         const CellsResult r = sort_cells(keys, tmp, M, shape, cnt, rank, part, cb, flag, bar, G,
-                                         &passed, info, wsum, &s_ok);
+                                         &passed, info, &wcnt[0][0], wsum, &s_ok);
         if (r != kCellsCrowded) return;
     }
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -1,6 +1,7 @@
 """GPU parity of rk_sort_device on key lists that no one search gives: keys
 outside the fields that the text length and the pattern count allow, and keys
-that occur more than once."""
+that occur more than once; and lists whose keys lie close together, which are
+sorted by the radix passes."""
 
 import numpy as np
 import pytest
@@ -87,3 +88,49 @@ def test_equal_keys(m, copies):
     keys = rng.permutation(np.repeat(own, copies)[:m])
     for spare in (0, 3000):
         assert np.array_equal(sort_keys(keys, n, k, spare), np.sort(keys)), spare
+
+
+def clumped(m, n, k, per_cell, rng):
+    """About m distinct keys with about per_cell to each 2^15 offsets of an id."""
+    span = int(min(n, max(64, m * 2**15 // (k * per_cell))))
+    keys = rng.integers(0, k, m).astype(np.uint64) << np.uint64(40)
+    keys |= (rng.integers(0, span, m) + (n - span) // 2).astype(np.uint64)
+    return rng.permutation(np.unique(keys))
+
+
+@pytest.mark.parametrize("per_cell", [8, 90, 110, 130, 500, 5000])
+@pytest.mark.parametrize("m", [2049, 5000, 300_001, 5_000_000])
+def test_clumped_keys(m, per_cell):
+    """On both sides of the mean cell size above which the radix passes run."""
+    n, k = 1 << 30, 100
+    keys = clumped(m, n, k, per_cell, np.random.default_rng(m + per_cell))
+    assert np.array_equal(sort_keys(keys, n, k, 1000), np.sort(keys))
+
+
+def test_clumped_keys_take_no_longer_than_the_passes():
+    """A few hundred keys to a cell: the radix passes take about twice as long as
+    cells do for evenly spread keys; comparing within the cells, six times."""
+    n, k, m = 1 << 30, 100, 5_000_000
+    rng = np.random.default_rng(3)
+    table = rk.rk_build([b"%06d" % i for i in range(k)])
+    try:
+        wsb = rk.rk_workspace_bytes(table, m)  # m: the most there are
+        ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+        took = []
+        for keys in (clumped(m, n, k, 1, rng), clumped(m, n, k, 700, rng)):
+            src = torch.from_numpy(keys.view(np.int64)).cuda()
+            d = torch.empty_like(src)
+            info = torch.tensor([src.numel(), 0], dtype=torch.int64, device="cuda")
+            best = 1e9
+            for _ in range(8):
+                d.copy_(src)
+                a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                a.record()
+                rk.rk_sort_device(table, n, d, src.numel(), info, ws, wsb)
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b))
+            took.append(best)
+        assert took[1] < 4 * took[0], took
+    finally:
+        rk.rk_destroy(table)
