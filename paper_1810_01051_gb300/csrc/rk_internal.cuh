@@ -58,17 +58,16 @@ struct alignas(16) LenRun {
 };
 constexpr uint32_t kManyPids = 0xFFFFFFFFu;
 
-// One slot of the sample map: a 4-byte gram (little-endian), the set of
-// offsets j (bit j, j < 4) at which it starts in some pattern (0 = empty), and,
-// when it occurs at one offset and after one prefix only, that prefix's slot
-// of the prefix map (else kNoSlot).
-struct alignas(16) SampSlot {
+// One slot of the sample map: a 4-byte gram (little-endian) and, in `at`, the set
+// of offsets j (bit j, j < 4) at which it starts in some pattern (0 = empty) and
+// above it, when it occurs at one offset and after one prefix only, that prefix's
+// slot of the prefix map (else kNoSlot).
+struct alignas(8) SampSlot {
     uint32_t key;
-    uint32_t mask;
-    uint32_t gi;
-    uint32_t pad;
+    uint32_t at;
 };
-constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
+constexpr uint32_t kSampOffsets = 4;
+constexpr uint32_t kNoSlot = (1u << (32 - kSampOffsets)) - 1u;
 
 // Bit of `ext` for four bytes read as a little-endian word.
 __host__ __device__ __forceinline__ uint32_t ext_bit(uint32_t w) {

@@ -261,9 +261,16 @@ __device__ __forceinline__ uint64_t cand_pack(uint64_t x, uint32_t slot, uint32_
 }
 constexpr uint32_t kCandBuf = kMatchCap / 2;     // 16-byte candidates in a warp's match buffer
 
-// The prefix-map slot whose lengths apply to a window whose bytes 0..7 are v
-// (little-endian): exact prefix, and a length below q + 4 or the next four
-// bytes in the slot's fingerprint set; -1 if none.
+// Whether a length of slot g applies to a window with its prefix and bytes 0..7 v
+// (little-endian): one below q + 4, or the next four bytes are in the slot's
+// fingerprint set.
+__device__ __forceinline__ bool gram_applies(const WinCtx &C, const GramSlot &g, uint64_t v) {
+    const bool ext_ok = (g.ext >> ext_bit((uint32_t)(v >> (8u * C.q)))) & 1u;
+    return ext_ok || (g.count & kGramShort);
+}
+
+// The prefix-map slot whose lengths apply to a window whose bytes 0..7 are v:
+// exact prefix and gram_applies; -1 if none.
 __device__ __forceinline__ int gram_lookup_v8(const WinCtx &C, uint64_t v) {
     const uint32_t key = C.q == 4 ? (uint32_t)v : (uint32_t)v & ((1u << (8u * C.q)) - 1u);
     const uint32_t gmask = (1u << C.gram_bits) - 1u;
@@ -271,10 +278,7 @@ __device__ __forceinline__ int gram_lookup_v8(const WinCtx &C, uint64_t v) {
     for (;;) {
         const GramSlot g = C.s2.grams[idx];
         if (g.count == 0) return -1;
-        if (g.key == key) {
-            const bool ext_ok = (g.ext >> ext_bit((uint32_t)(v >> (8u * C.q)))) & 1u;
-            return ext_ok || (g.count & kGramShort) ? (int)idx : -1;
-        }
+        if (g.key == key) return gram_applies(C, g, v) ? (int)idx : -1;
         idx = (idx + 1) & gmask;
     }
 }
@@ -339,10 +343,10 @@ __device__ __forceinline__ void cand_overflow(const WinCtx &C, const WarpCtx &w,
     probe_slot<true>(C, w, buf, (uint32_t)(x + C.mis - u0), x, cand_slot(e), cand_class(e));
 }
 
-// Stage 2a for the window at pos of the tile at u0 (known: its prefix-map slot,
-// when the sample map names it); a candidate is queued in
-// the warp's buffer (w.mbuf as kCandBuf 16-byte entries), or offered to the
-// list when that is full.
+// Stage 2a for the window at pos of the tile at u0 (known: the one prefix-map slot
+// it can have, when the sample map names it: read and checked without a search); a
+// candidate is queued in the warp's buffer (w.mbuf as kCandBuf 16-byte entries),
+// or offered to the list when that is full.
 __device__ __forceinline__ void cand_window(const WinCtx &C, const WarpCtx &w, const CandList &cc,
                                             const uint8_t *buf, uint32_t pos, uint64_t u0,
                                             uint32_t known = kNoSlot) {
@@ -354,7 +358,9 @@ __device__ __forceinline__ void cand_window(const WinCtx &C, const WarpCtx &w, c
         gi = gram_lookup(C, buf, pos, &v8);
         if (gi < 0) return;
     } else {
-        v8 = ld8(buf, pos);
+        v8 = ld8(buf, pos);  // (sampled: q is 4)
+        const GramSlot g = C.s2.grams[known];
+        if (g.key != (uint32_t)v8 || !gram_applies(C, g, v8)) return;
     }
     const ulonglong2 c = make_ulonglong2(cand_pack(ua - C.mis, (uint32_t)gi, kLenAll), v8);
     const uint32_t s = atomicAdd(w.mcount, 1u);
@@ -560,10 +566,10 @@ __device__ __forceinline__ void samp_window(const WinCtx &C, const WarpCtx &w, c
     uint32_t offs = 0, known = kNoSlot;
     for (;;) {
         const SampSlot e = C.s2.smap[idx];
-        if (e.mask == 0) return;  // a false positive of the bit set
+        if (e.at == 0) return;  // a false positive of the bit set
         if (e.key == key) {
-            offs = e.mask;
-            known = e.gi;
+            offs = e.at & ((1u << kSampOffsets) - 1u);
+            known = e.at >> kSampOffsets;
             break;
         }
         idx = (idx + 1) & smask;

@@ -399,13 +399,13 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
         for (auto &kv : offs) skeys.push_back(kv.first);
         std::sort(skeys.begin(), skeys.end());
         smap_bits = std::max<uint32_t>(4, ceil_log2(2ull * skeys.size()));
-        smap.assign(1ull << smap_bits, SampSlot{0, 0, 0, 0});
+        smap.assign(1ull << smap_bits, SampSlot{0, 0});
         const uint32_t smask = (1u << smap_bits) - 1;
         for (uint32_t key : skeys) {
             uint32_t idx = (key * kGramMult) >> (32 - smap_bits);
-            while (smap[idx].mask) idx = (idx + 1) & smask;
+            while (smap[idx].at) idx = (idx + 1) & smask;
             const Gram &g = offs[key];
-            smap[idx] = SampSlot{key, g.mask, g.one ? g.gi : kNoSlot, 0};
+            smap[idx] = SampSlot{key, ((g.one ? g.gi : kNoSlot) << kSampOffsets) | g.mask};
         }
         // the same layout choice as the prefix bit set, for this key set; a
         // flat one tests three bits per gram (stage 1 tests 4x fewer positions)
@@ -455,7 +455,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     size_t o_grams = b.add(grams.size() * sizeof(GramSlot));
     size_t o_runs = b.add(gram_runs.size() * sizeof(LenRun) + sizeof(LenRun));
     size_t o_pbytes = b.add(packed + 16);
-    size_t o_smap = b.add(smap.size() * sizeof(SampSlot) + 16);
+    size_t o_smap = b.add(smap.size() * sizeof(SampSlot) + 8);
     // the hash tables of the lengths and what goes with them: with a prefilter
     // only windows whose prefix and length several patterns share get there,
     // so these stay in global memory
