@@ -19,6 +19,7 @@
 
 #include "rk_internal.cuh"
 #include "rk_layout.cuh"
+#include "rk_limit.h"
 
 namespace rk {
 namespace {
@@ -449,6 +450,10 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
         }
     }
 
+    const SetParts parts{k, packed, D, gram_runs.size(), slots.size(), lengths.size(), lmax,
+                         smap.size(), simg.size() * 4, (rimg.size() + rside.size()) * 4};
+    if (!set_fits(parts)) return RK_EINVAL;
+
     // ---- one device allocation --------------------------------------------
     Blob b;
     size_t o_filter = b.add(fimg.size() * 4 + 16);
@@ -485,7 +490,6 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     if (!rimg.empty()) memcpy(hb + o_rfilter, rimg.data(), rimg.size() * 4);
     if (!rside.empty()) memcpy(hb + o_rfilter + rimg.size() * 4, rside.data(), rside.size() * 4);
 
-    if (b.bytes.size() - o_grams > 0xFFFFFFFFull) return RK_EINVAL;  // tables above 4 GiB
     TableBlob &tb = *out;
     tb.o_filter = o_filter;
     tb.o_grams = o_grams;
@@ -521,7 +525,8 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     d.rfilter_bytes = (uint32_t)((rimg.size() + rside.size()) * 4);
     d.rf_side_off = rside.empty() ? 0u : (uint32_t)(rimg.size() * 4);
     d.rf_shift = rstep ? 30 - (rbits - 5) : 0;
-    d.s2_bytes = (uint32_t)((mode == kFilterNone ? o_sfilter : o_ghdr) - o_grams);
+    d.s2_bytes = (uint32_t)std::min<size_t>(
+        (mode == kFilterNone ? o_sfilter : o_ghdr) - o_grams, UINT32_MAX);
     d.gram_mult = gram_mult;
     tb.n_grams = D;
     tb.filter_log2_bits = mode == kFilterNone ? 0 : fbits;
