@@ -135,7 +135,7 @@ struct DevTable {
     // The prefix map, its runs, the pattern bytes and the sample map lie in
     // [s2_base, s2_base + s2_bytes): the survivor-stage tables, which the scan
     // kernel may copy to shared memory as one block.  Without a prefilter
-    // (kFilterNone) the block goes on to the lengths' hash tables.
+    // (kFilterNone) the block is the pattern bytes and the lengths' hash tables.
     const uint8_t *s2_base;
     uint32_t s2_bytes;
 };
@@ -206,7 +206,7 @@ namespace rk {
 // offsets of its parts; `meta` holds the device view's non-pointer fields.
 struct TableBlob {
     std::vector<uint8_t> bytes;
-    size_t o_filter = 0, o_grams = 0, o_runs = 0, o_ghdr = 0, o_slots = 0, o_gpids = 0,
+    size_t o_filter = 0, o_s2 = 0, o_grams = 0, o_runs = 0, o_ghdr = 0, o_slots = 0, o_gpids = 0,
            o_pbytes = 0, o_poff = 0, o_plen = 0, o_lens = 0, o_sfilter = 0, o_smap = 0,
            o_rfilter = 0;
     DevTable meta{};

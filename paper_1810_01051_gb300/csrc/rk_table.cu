@@ -254,6 +254,38 @@ bool make_role_filter(const uint8_t *patterns, const std::vector<uint64_t> &src_
 
 }  // namespace
 
+// A place for every prefix (ascending) in a map of 2^bits slots, open addressing
+// from (key * m) >> (32 - bits); m: of a few multipliers the one with the fewest
+// probes.  Returns m.
+static uint32_t place_prefixes(const std::vector<uint32_t> &keys, uint32_t bits,
+                               std::vector<uint32_t> *slot) {
+    const uint32_t mask = (1u << bits) - 1;
+    uint32_t mult = kGramMult, best = UINT32_MAX;
+    std::vector<uint8_t> used;
+    std::vector<uint32_t> at(keys.size());
+    for (uint32_t i = 0, m = kGramMult; i < (keys.size() <= 1024 ? 8u : 1u) && best > 1;
+         ++i, m = m * 5 + 2) {
+        used.assign(1ull << bits, 0);
+        uint32_t longest = 0;  // probes of the last key found
+        for (size_t j = 0; j < keys.size(); ++j) {
+            uint32_t idx = (keys[j] * m) >> (32 - bits), probes = 1;
+            for (; used[idx]; ++probes) idx = (idx + 1) & mask;
+            used[idx] = 1;
+            at[j] = idx;
+            longest = std::max(longest, probes);
+        }
+        if (longest < best) {
+            best = longest;
+            mult = m;
+            *slot = at;
+        }
+    }
+    return mult;
+}
+
+// Least size (log2 slots) of the map of D prefixes: one slot in two free.
+static uint32_t dense_bits(uint32_t D) { return std::max<uint32_t>(4, ceil_log2(2ull * D)); }
+
 // Serialise the pattern table of one pattern set into a host image; every
 // part is 256-byte aligned and the image ends on a 256-byte boundary.
 int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32_t base_log2,
@@ -303,34 +335,18 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     uint32_t D = (uint32_t)gram_keys.size();
     // A warp's lookup takes as many probes as its unluckiest lane, so the map
     // is sparse: one slot in eight used (up to 16 KiB), else one in four (one
-    // in two above 2^19 prefixes: a listed candidate holds a slot in 22 bits),
-    // and the multiplier is the one of a few with the fewest probes.
+    // in two above 2^19 prefixes: a listed candidate holds a slot in 22 bits).
+    // shrink_map makes it denser where shared memory is short.
     const uint64_t sparse = D <= 128 ? 8 : D <= (1u << 19) ? 4 : 2;
-    uint32_t gram_bits = std::max<uint32_t>(4, ceil_log2(sparse * D));
+    const uint32_t gram_bits = std::max<uint32_t>(4, ceil_log2(sparse * D));
     std::vector<GramSlot> grams(1ull << gram_bits, GramSlot{0, 0, 0, 0});
     std::vector<LenRun> gram_runs;
     const uint32_t mask = (1u << gram_bits) - 1;
-    uint32_t gram_mult = kGramMult, best = UINT32_MAX;
-    std::vector<uint8_t> used;
-    for (uint32_t i = 0, m = kGramMult; i < (D <= 1024 ? 8u : 1u) && best > 1;
-         ++i, m = m * 5 + 2) {
-        used.assign(1ull << gram_bits, 0);
-        uint32_t longest = 0;  // probes of the last key found
-        for (uint32_t key : gram_keys) {
-            uint32_t idx = (key * m) >> (32 - gram_bits), probes = 1;
-            for (; used[idx]; ++probes) idx = (idx + 1) & mask;
-            used[idx] = 1;
-            longest = std::max(longest, probes);
-        }
-        if (longest < best) {
-            best = longest;
-            gram_mult = m;
-        }
-    }
-    for (uint32_t key : gram_keys) {
+    std::vector<uint32_t> gram_at;
+    const uint32_t gram_mult = place_prefixes(gram_keys, gram_bits, &gram_at);
+    for (uint32_t g = 0; g < D; ++g) {
+        const uint32_t key = gram_keys[g];
         const auto &v = gram_to_lens[key];
-        uint32_t idx = (key * gram_mult) >> (32 - gram_bits);
-        while (grams[idx].count) idx = (idx + 1) & mask;
         const uint32_t shorts = v.front().first < q + 4 ? kGramShort : 0u;  // v ascends
         const uint32_t first = (uint32_t)gram_runs.size();
         uint32_t n_runs = 0;
@@ -344,7 +360,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
             ++n_runs;
             i = j;
         }
-        grams[idx] = GramSlot{key, first, n_runs | shorts, gram_ext[key]};
+        grams[gram_at[g]] = GramSlot{key, first, n_runs | shorts, gram_ext[key]};
     }
 
     // ---- stage-1 bit set ---------------------------------------------------
@@ -492,6 +508,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
 
     TableBlob &tb = *out;
     tb.o_filter = o_filter;
+    tb.o_s2 = mode == kFilterNone ? o_pbytes : o_grams;
     tb.o_grams = o_grams;
     tb.o_runs = o_runs;
     tb.o_ghdr = o_ghdr;
@@ -526,7 +543,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     d.rf_side_off = rside.empty() ? 0u : (uint32_t)(rimg.size() * 4);
     d.rf_shift = rstep ? 30 - (rbits - 5) : 0;
     d.s2_bytes = (uint32_t)std::min<size_t>(
-        (mode == kFilterNone ? o_sfilter : o_ghdr) - o_grams, UINT32_MAX);
+        (mode == kFilterNone ? o_sfilter : o_ghdr) - tb.o_s2, UINT32_MAX);
     d.gram_mult = gram_mult;
     tb.n_grams = D;
     tb.filter_log2_bits = mode == kFilterNone ? 0 : fbits;
@@ -534,6 +551,43 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     tb.rfilter_log2_bits = rstep ? rbits : 0;
     tb.bytes = std::move(b.bytes);
     return RK_OK;
+}
+
+// Lay the prefix map of an image out in 2^bits slots, fewer than it has; every
+// part after it moves up.
+void shrink_map(TableBlob *b, uint32_t bits) {
+    DevTable &d = b->meta;
+    const uint32_t n = 1u << d.gram_bits;
+    const GramSlot *old = reinterpret_cast<const GramSlot *>(b->bytes.data() + b->o_grams);
+    std::vector<std::pair<uint32_t, uint32_t>> used;  // key, slot
+    for (uint32_t i = 0; i < n; ++i)
+        if (old[i].count) used.emplace_back(old[i].key, i);
+    std::sort(used.begin(), used.end());
+    std::vector<uint32_t> keys, at, moved(n);
+    for (const auto &u : used) keys.push_back(u.first);
+    d.gram_mult = place_prefixes(keys, bits, &at);
+    std::vector<GramSlot> now(1ull << bits, GramSlot{0, 0, 0, 0});
+    for (size_t i = 0; i < used.size(); ++i) {
+        now[at[i]] = old[used[i].second];
+        moved[used[i].second] = at[i];
+    }
+    if (d.sample == 4) {  // the sample map names slots
+        SampSlot *s = reinterpret_cast<SampSlot *>(b->bytes.data() + b->o_smap);
+        for (uint32_t i = 0; i < 1u << d.smap_bits; ++i)
+            if (s[i].at && s[i].at >> kSampOffsets != kNoSlot)
+                s[i].at = (moved[s[i].at >> kSampOffsets] << kSampOffsets) |
+                          (s[i].at & ((1u << kSampOffsets) - 1u));
+    }
+    const size_t cut = (n - now.size()) * sizeof(GramSlot);  // a multiple of 256
+    memcpy(b->bytes.data() + b->o_grams, now.data(), now.size() * sizeof(GramSlot));
+    const auto end = b->bytes.begin() + b->o_grams + now.size() * sizeof(GramSlot);
+    b->bytes.erase(end, end + cut);
+    for (size_t *o : {&b->o_runs, &b->o_ghdr, &b->o_slots, &b->o_gpids, &b->o_pbytes, &b->o_poff,
+                      &b->o_plen, &b->o_lens, &b->o_sfilter, &b->o_smap, &b->o_rfilter})
+        *o -= cut;
+    d.gram_bits = bits;
+    if (d.filter_mode == kFilterNone) b->o_s2 -= cut;
+    else d.s2_bytes -= (uint32_t)cut;
 }
 
 // Point the device view of a table at its image placed at device address dm.
@@ -552,7 +606,7 @@ void bind_blob(DevTable *d, const TableBlob &b, const uint8_t *dm) {
     d->smap = (const SampSlot *)(dm + b.o_smap);
     d->sfilter = (const uint32_t *)(dm + b.o_sfilter);
     d->rfilter = (const uint32_t *)(dm + b.o_rfilter);
-    d->s2_base = dm + b.o_grams;
+    d->s2_base = dm + b.o_s2;
 }
 
 }  // namespace rk
@@ -639,13 +693,21 @@ int plan_with(const uint8_t *patterns, const uint32_t *lens, uint32_t k, const O
         return role ? rf_smem_layout(fbytes, s2b, sv, st, tl, halo).total
                     : smem_layout(fbytes, s2b, warps, st, tl, halo).total;
     };
+    // A denser prefix map (shrink_map) comes before fewer stages, and both before the
+    // tables in L2: 64 MiB of words and 300 patterns of 8..64 letters, every position
+    // tested: copied 87 us, in L2 with the sparse map 115; 4 MiB and 600 patterns of
+    // 4..32 without a prefilter 1583 and 1830 us.
     uint32_t s2 = 0;
-    if (s2_total <= limit) {
-        if (total((uint32_t)s2_total, stages, tile) <= limit) {
-            s2 = (uint32_t)s2_total;
-        } else if (total((uint32_t)s2_total, 2, tile) <= limit) {
-            s2 = (uint32_t)s2_total;
-            stages = 2;
+    const uint32_t sparse = tb->meta.gram_bits,
+                   dense = tb->meta.filter_mode == kFilterNone ? sparse : dense_bits(tb->n_grams);
+    const uint64_t cut1 = sizeof(GramSlot) << sparse;
+    for (const uint32_t st : {stages, 2u}) {
+        for (uint32_t bits = sparse; !s2 && bits >= dense; --bits) {
+            const uint64_t size = s2_total - (cut1 - (sizeof(GramSlot) << bits));
+            if (size > limit || total((uint32_t)size, st, tile) > limit) continue;
+            if (bits < sparse) shrink_map(tb, bits);
+            s2 = (uint32_t)size;
+            stages = st;
         }
     }
     uint32_t bytes = total(s2, stages, tile);

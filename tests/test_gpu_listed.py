@@ -9,7 +9,8 @@ import oracle
 
 pytestmark = pytest.mark.gpu
 
-from gpu_util import assert_same, keys_to_pairs, require_gpu, to_device  # noqa: E402
+from gpu_util import (assert_same, gpu_search, keys_to_pairs, require_gpu,  # noqa: E402
+                      to_device)
 from paper_1810_01051_gb300 import rk  # noqa: E402
 
 torch = pytest.importorskip("torch")
@@ -66,3 +67,27 @@ def test_listed_windows_start_with_a_prefix(run, many):
         got, listed = listed_scan(pats, text, mis, role_step=1)
         assert_same(got, expect, f"mis {mis}")
         assert expect[0].size <= listed <= with_prefix
+
+
+@pytest.mark.parametrize("opts,lmin,lmax,counts", [
+    (dict(), 8, 64, (120, 250, 290, 310, 330)),
+    (dict(role_step=1), 8, 64, (80, 200, 300, 336)),
+    (dict(role_step=1, sample=1), 8, 40, (300, 420)),
+    (dict(role_step=1), 3, 12, (300, 500)),
+    (dict(filter=rk.RK_FILTER_NONE), 4, 32, (40, 520)),
+])
+def test_every_density_of_the_prefix_map(opts, lmin, lmax, counts):
+    """Sets whose map is sparse, denser or as dense as it gets, so that their
+    tables still fit shared memory: searched in the scan and through the list."""
+    rng = np.random.default_rng(lmin + lmax)
+    n = 60_000 if "filter" in opts else 300_000
+    text = rng.choice(np.frombuffer(b"etaoinsh rdlcum", np.uint8), n)
+    for k in counts:
+        at = rng.integers(0, n - lmax, k)
+        pats = [text[a:a + int(L)].tobytes() for a, L in zip(at, rng.integers(lmin, lmax + 1, k))]
+        expect = oracle.rabin_karp(text, pats)
+        if "filter" not in opts:
+            got, listed = listed_scan(pats, text, 5, **opts)
+            assert_same(got, expect, f"listed, {k}")
+            assert listed > 0
+        assert_same(gpu_search(pats, text, 5, **opts), expect, f"in the scan, {k}")
