@@ -162,16 +162,26 @@ namespace {
 // 8 us whatever the text, the scan's own comparisons more per survivor.
 //   - survivor tables in shared memory: prefix filters always (100 words of
 //     3..12, 64 MiB: 150 us in the scan, 180 us with the list, 256 MiB: 562 and
-//     624 us), role filters up to kInScanRoles bytes (100 words of 4..32, 1 MiB:
-//     14 and 22 us, 32 MiB: 36 and 40, 256 MiB: 171 and 165; DNA probes of
-//     25..800, 32 MiB: 86 and 92, 64 MiB: 144 and 129);
+//     624 us).  Role filters, whose few survivor warps a crowd of survivors holds
+//     up, where few are expected (rk_table::survivors, s): s up to kInScanMost and
+//     s^2 n up to kInScanMany, n up to kInScanRoles.  In the scan / with the list,
+//     at 1 MiB, 8 MiB, 48 MiB: 100 words of 4..32 (s 0.016) 16 / 23, 23 / 29,
+//     36 / 46 us; 8 DNA probes of 16 (0.034) 16 / 24, 24 / 29, 43 / 48; 16 of them
+//     (0.066) 20 / 29, 39 / 42, 92 / 89; 300 words of 4..8 (0.15) 38 / 38, 139 / 124,
+//     491 / 361; 64 probes (0.22) 101 / 87, 323 / 228, 1315 / 749; 256 (0.63)
+//     243 / 138, 1026 / 390, 4423 / 1307;
 //   - tables in L2: only sampled ones (the scan then tests every position) up
 //     to kInScanSampled (10,000 signatures, 1 MiB: 16 and 23 us, 8 MiB: 32 and
 //     32); role filters lose from 1 MiB on (1000 signatures: 28 and 25 us).
 constexpr uint64_t kInScanRoles = 48ull << 20, kInScanSampled = 4ull << 20;
+constexpr double kInScanMost = 0.2, kInScanMany = 0.06 * (1 << 20);
 
 bool complete_in_scan(const rk_table *t, uint64_t n) {
-    if (t->tune.s2_smem && t->dev.sample != 4) return !t->dev.rf_step || n <= kInScanRoles;
+    if (t->tune.s2_smem && t->dev.sample != 4) {
+        const double s = t->survivors;
+        return !t->dev.rf_step ||
+               (n <= kInScanRoles && s <= kInScanMost && s * s * (double)n <= kInScanMany);
+    }
     return t->dev.sample == 4 && n <= kInScanSampled;
 }
 

@@ -160,6 +160,7 @@ struct rk_table {
     rk::DevTable dev{};
     rk::Tuning tune{};
     uint32_t n_grams = 0;
+    double survivors = 0;  // see TableBlob
     uint32_t filter_log2_bits = 0;
     uint32_t sfilter_log2_bits = 0;
     uint32_t rfilter_log2_bits = 0;
@@ -211,6 +212,10 @@ struct TableBlob {
            o_rfilter = 0;
     DevTable meta{};
     uint32_t n_grams = 0, filter_log2_bits = 0, sfilter_log2_bits = 0, rfilter_log2_bits = 0;
+    // the chance that a window of a text made of the patterns' bytes, as often as
+    // they have them, starts with a prefix; a prefix of a pattern under 7 bytes, which
+    // a role filter tells by four bytes alone, counts eight times
+    double survivors = 0;
 };
 
 // sample_opt: rk_build_opts.sample (1: no sampled structures); role_opt:

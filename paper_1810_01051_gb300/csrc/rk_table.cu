@@ -369,6 +369,18 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     if (!make_filter(gram_keys, filter_opt, filter_bits_opt, false, &mode, &fbits, &fimg, &fmask))
         return RK_EINVAL;
 
+    // ---- windows that survive in a text of the patterns' own bytes ----------
+    double survivors = 0;
+    {
+        double freq[256] = {};
+        for (uint64_t i = 0; i < acc; ++i) freq[patterns[i]] += 1.0 / (double)acc;
+        for (uint32_t key : gram_keys) {
+            double p = gram_to_lens[key].front().first < 7 ? 8 : 1;
+            for (uint32_t j = 0; j < q; ++j) p *= freq[key >> (8 * j) & 0xFFu];
+            survivors += p;
+        }
+    }
+
     // ---- role filter: sampled grams with their roles ------------------------
     std::vector<uint32_t> rimg, rside;
     uint32_t rstep = 0, rbits = 0;
@@ -546,6 +558,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
         (mode == kFilterNone ? o_sfilter : o_ghdr) - tb.o_s2, UINT32_MAX);
     d.gram_mult = gram_mult;
     tb.n_grams = D;
+    tb.survivors = survivors;
     tb.filter_log2_bits = mode == kFilterNone ? 0 : fbits;
     tb.sfilter_log2_bits = sampled ? sbits : 0;
     tb.rfilter_log2_bits = rstep ? rbits : 0;
@@ -820,6 +833,7 @@ extern "C" int rk_build(const uint8_t *patterns, const uint32_t *lens, uint32_t 
     bind_blob(&t->dev, tb, (const uint8_t *)t->d_mem);
     t->tune = tune;
     t->n_grams = tb.n_grams;
+    t->survivors = tb.survivors;
     t->filter_log2_bits = tb.filter_log2_bits;
     t->sfilter_log2_bits = tb.sfilter_log2_bits;
     t->rfilter_log2_bits = tb.rfilter_log2_bits;
