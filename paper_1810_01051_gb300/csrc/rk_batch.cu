@@ -29,6 +29,8 @@ struct BatchItem {
     uint64_t n;
 };
 
+constexpr uint32_t kMaxBatchS2 = 1u << 17;  // survivor tables per stage, at most
+
 struct BatchDesc {
     uint32_t n_items, n_chunks;
     uint32_t work_counter;
@@ -348,7 +350,7 @@ extern "C" int rk_tableset_build(uint32_t n_tables, const uint8_t *patterns, con
     std::vector<TableBlob> blobs(n_tables);
     std::vector<size_t> at(n_tables);
     size_t size = 0;
-    uint64_t pat_off = 0, byte_off = 0;
+    uint64_t pat_off = 0, byte_off = 0, most = 0;
     rk_tableset *ts = new (std::nothrow) rk_tableset();
     if (!ts) return RK_ENOMEM;
     ts->n_tables = n_tables;
@@ -368,14 +370,21 @@ extern "C" int rk_tableset_build(uint32_t n_tables, const uint8_t *patterns, con
         if (rc) { delete ts; return rc; }
         for (uint32_t j = 0; j < k; ++j) byte_off += lens[pat_off + j];
         pat_off += k;
-        at[i] = size;
-        size += blobs[i].bytes.size();  // each blob is a multiple of 256 bytes
+        most = std::max(most, blobs[i].counted_s2);
         const DevTable &m = blobs[i].meta;
         ts->max_filter_bytes = std::max(ts->max_filter_bytes, m.filter_bytes);
-        ts->max_s2_bytes = std::max(ts->max_s2_bytes, m.s2_bytes);
         ts->max_lmax = std::max(ts->max_lmax, m.lmax);
         ts->max_patterns = std::max(ts->max_patterns, k);
         if (m.q != 4) ts->all_q4 = false;
+    }
+    // A batch may reserve the largest set's survivor tables per stage: a prefix map
+    // that would make it larger than the sets count for gets denser, so that no launch
+    // shape stops fitting for the sake of a sparse one.
+    for (uint32_t i = 0; i < n_tables; ++i) {
+        if (most <= kMaxBatchS2) shrink_s2(&blobs[i], most);
+        at[i] = size;
+        size += blobs[i].bytes.size();  // each blob is a multiple of 256 bytes
+        ts->max_s2_bytes = std::max(ts->max_s2_bytes, blobs[i].meta.s2_bytes);
     }
     if (byte_off) ts->bytes.assign(patterns, patterns + byte_off);
     if (pat_off) ts->lens.assign(lens, lens + pat_off);
@@ -578,7 +587,7 @@ int resolve(rk_batch *b, rk_batch_opts *o) {
         o->tile_bytes > kMaxTileBytes || o->stages < 2 || o->stages > 8 || o->ctas_per_sm < 1 ||
         o->ctas_per_sm > 8)
         return RK_EINVAL;
-    if (o->s2_in_smem && b->ts->max_s2_bytes > (1u << 17)) return RK_EINVAL;
+    if (o->s2_in_smem && b->ts->max_s2_bytes > kMaxBatchS2) return RK_EINVAL;
     uint32_t limit = 0;
     int rc = smem_limit(b, *o, &limit);
     if (rc) return rc;

@@ -216,6 +216,7 @@ struct TableBlob {
     // they have them, starts with a prefix; a prefix of a pattern under 7 bytes, which
     // a role filter tells by four bytes alone, counts eight times
     double survivors = 0;
+    uint64_t counted_s2 = 0;  // what the set's tables other than bit sets count for (set_bytes)
 };
 
 // sample_opt: rk_build_opts.sample (1: no sampled structures); role_opt:
@@ -224,6 +225,7 @@ struct TableBlob {
 int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32_t base_log2,
                uint32_t filter_opt, uint32_t filter_bits_opt, uint32_t sample_opt,
                uint32_t role_opt, TableBlob *out);
+void shrink_s2(TableBlob *b, uint64_t most);
 void bind_blob(DevTable *d, const TableBlob &b, const uint8_t *dev_base);
 
 // Candidate list of a scan whose survivors are verified in a second pass

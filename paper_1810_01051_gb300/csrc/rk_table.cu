@@ -559,6 +559,10 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     d.gram_mult = gram_mult;
     tb.n_grams = D;
     tb.survivors = survivors;
+    // (a set without its two bit sets, each of which counts for a part at least)
+    SetParts tables = parts;
+    tables.sample_filter_bytes = tables.role_filter_bytes = 0;
+    tb.counted_s2 = set_bytes(tables) - 2 * 256;
     tb.filter_log2_bits = mode == kFilterNone ? 0 : fbits;
     tb.sfilter_log2_bits = sampled ? sbits : 0;
     tb.rfilter_log2_bits = rstep ? rbits : 0;
@@ -568,7 +572,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
 
 // Lay the prefix map of an image out in 2^bits slots, fewer than it has; every
 // part after it moves up.
-void shrink_map(TableBlob *b, uint32_t bits) {
+static void shrink_map(TableBlob *b, uint32_t bits) {
     DevTable &d = b->meta;
     const uint32_t n = 1u << d.gram_bits;
     const GramSlot *old = reinterpret_cast<const GramSlot *>(b->bytes.data() + b->o_grams);
@@ -601,6 +605,18 @@ void shrink_map(TableBlob *b, uint32_t bits) {
     d.gram_bits = bits;
     if (d.filter_mode == kFilterNone) b->o_s2 -= cut;
     else d.s2_bytes -= (uint32_t)cut;
+}
+
+// Make the prefix map denser until the survivor tables take at most `most` bytes,
+// if they can.
+void shrink_s2(TableBlob *b, uint64_t most) {
+    if (b->meta.filter_mode == kFilterNone) return;  // no map among them
+    const uint32_t sparse = b->meta.gram_bits;
+    for (uint32_t bits = sparse; bits >= dense_bits(b->n_grams); --bits)
+        if (b->meta.s2_bytes - ((sizeof(GramSlot) << sparse) - (sizeof(GramSlot) << bits)) <= most) {
+            if (bits < sparse) shrink_map(b, bits);
+            return;
+        }
 }
 
 // Point the device view of a table at its image placed at device address dm.
