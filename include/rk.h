@@ -434,7 +434,7 @@ int rk_batch_read(const rk_batch *b, uint64_t *h_keys, uint64_t key_cap, uint64_
 /* Autotuner (the paper's threads-per-block sweep of Table 1, automated):
  * time up to max_candidates launch shapes (tile size, warps, stages, CTAs
  * per SM, survivor-table placement; 0 = all that fit, else an even spread of
- * them), each `reps` times (0: 3) on the current batch, keep the fastest and
+ * them; the one in use is always among them), each `reps` times (0: 3) on the current batch, keep the fastest and
  * re-capture the graph.  Only the scan is timed (the sort's work does not
  * depend on the shape).  *best_ms (may be NULL) gets the best scan time, or
  * -1 when no shape could run (the previous shape is kept).

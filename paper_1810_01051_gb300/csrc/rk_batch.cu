@@ -14,6 +14,7 @@
 #include <new>
 
 #include "rk_scan_body.cuh"
+#include "rk_shapes.h"
 #include "rk_sortws.cuh"
 
 namespace rk {
@@ -755,14 +756,7 @@ extern "C" int rk_batch_autotune(rk_batch *b, uint32_t max_candidates, uint32_t 
                         o.ctas_per_sm = cps;
                         if (resolve(b, &o) == RK_OK) cand.push_back(o);
                     }
-    if (max_candidates && cand.size() > max_candidates) {
-        // keep an even spread of the candidate list
-        std::vector<rk_batch_opts> pick;
-        for (uint32_t i = 0; i < max_candidates; ++i)
-            pick.push_back(cand[(size_t)i * cand.size() / max_candidates]);
-        cand.swap(pick);
-    }
-    cand.push_back(keep);
+    cand = pick_shapes(cand, max_candidates, keep);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
         if (e0) cudaEventDestroy(e0);
