@@ -372,8 +372,10 @@ typedef struct rk_batch_opts {
     uint64_t max_text_len;     /* longest text, >= 1 (sets offset_bits) */
     uint64_t max_total_bytes;  /* most text bytes in one batch */
     uint64_t capacity;         /* match keys per batch, < 2^32 */
-    /* launch shape; with all four 0: three CTAs of 8 warps per SM and 24 KiB tiles
-     * where their shared memory fits, else (and for any given alone) the defaults named */
+    /* launch shape; with all four 0, limits of many chunks (max_items + max_total_bytes /
+     * 96 KiB at least 27 per SM), tables that few windows survive (or texts under 8 KiB on
+     * average) and shared memory for it: three CTAs of 8 warps per SM and 24 KiB tiles;
+     * else (and for any given alone) the defaults named */
     uint32_t warps;            /* consumer warps per CTA (default 16) */
     uint32_t tile_bytes;       /* bytes per tile, multiple of 16, <= 65536 (default 32768) */
     uint32_t stages;           /* tiles in flight per CTA (default 2) */

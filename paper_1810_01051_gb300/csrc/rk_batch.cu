@@ -372,6 +372,7 @@ extern "C" int rk_tableset_build(uint32_t n_tables, const uint8_t *patterns, con
         for (uint32_t j = 0; j < k; ++j) byte_off += lens[pat_off + j];
         pat_off += k;
         most = std::max(most, blobs[i].counted_s2);
+        ts->survivors += blobs[i].survivors / n_tables;
         const DevTable &m = blobs[i].meta;
         ts->max_filter_bytes = std::max(ts->max_filter_bytes, m.filter_bytes);
         ts->max_lmax = std::max(ts->max_lmax, m.lmax);
@@ -565,11 +566,22 @@ int capture(rk_batch *b) {
 }
 
 int resolve(rk_batch *b, rk_batch_opts *o) {
-    // Three CTAs of 8 warps per SM where they fit: one tile's end (few survivors,
-    // a chain of reads from L2) overlaps the others' first stage.  1024 texts of
-    // 1 KiB..16 MiB 1485 -> 1378 us, 4096 of 1..64 KiB 111 -> 89 us, against one
-    // of 16 warps.
-    if (!o->warps && !o->tile_bytes && !o->stages && !o->ctas_per_sm) {
+    // Three CTAs of 8 warps per SM, where they fit, for batches of many chunks with
+    // few survivors: one tile's end (few survivors, a chain of reads from L2) overlaps
+    // the others' first stage, and a text's set-up the others' work.  One of 16 warps
+    // / three of 8: 4096 texts of 4 KiB 75 / 44 us, of 1..64 KiB 104 / 77, 1024 of
+    // 1 KiB..16 MiB 1168 / 1109.  A batch of few chunks leaves CTAs idle and the others
+    // with half the warps (64 texts of 64 KiB 26 / 32, 512 of them 44 / 50, 64 of 4 MiB
+    // 177 / 179): it needs kChunksPerCta for each.  Where many windows survive (DNA,
+    // 1..256 patterns, 0.4 by the tables' mean) the survivors' own work fills the SM,
+    // and only the set-up of very short texts still tells: 4096 of 4 KiB 733 / 466, of
+    // 64 KiB 2512 / 3080, 512 of 1 MiB 5207 / 6236 (1..64 patterns, 0.1: 1250 / 1291).
+    constexpr uint64_t kChunksPerCta = 9, kShortText = 8192;
+    constexpr double kFewSurvivors = 0.125;
+    const uint64_t chunks = o->max_items + o->max_total_bytes / (24576 * kTilesPerChunk);
+    if (!o->warps && !o->tile_bytes && !o->stages && !o->ctas_per_sm &&
+        chunks >= kChunksPerCta * 3 * (uint64_t)b->sm_count &&
+        (b->ts->survivors <= kFewSurvivors || o->max_total_bytes / o->max_items <= kShortText)) {
         rk_batch_opts c = *o;
         c.warps = 8;
         c.tile_bytes = 24576;

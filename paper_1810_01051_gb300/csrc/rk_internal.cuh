@@ -190,6 +190,7 @@ struct rk_tableset {
     const rk::DevTable *d_tables = nullptr;  // device array
     uint32_t filter_mode = rk::kFilterFlat;
     uint32_t max_filter_bytes = 0, max_s2_bytes = 0, max_lmax = 1, max_patterns = 0;
+    double survivors = 0;  // TableBlob::survivors, the tables' mean
     bool all_q4 = true;
     uint32_t base_log2 = 8;
     std::vector<uint32_t> npat;  // patterns per table

@@ -438,6 +438,8 @@ extern "C" int rk_server_create(const rk_tableset *ts, const rk_server_opts *opt
         bo.capacity = o.batch_capacity;
         bo.tile_bytes = o.tile_bytes;
         bo.warps = o.warps;
+        // most batches hold a few requests, far below these limits: one CTA per SM
+        bo.ctas_per_sm = 1;
         rc = rk_batch_create(ts, &bo, &e.b);
         if (!rc && (cudaStreamCreateWithFlags(&e.st, cudaStreamNonBlocking) != cudaSuccess ||
                     cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming) != cudaSuccess))

@@ -69,3 +69,41 @@ def test_shape_fits_and_matches(counts, lens, stages, warps, tile):
     finally:
         rk.rk_batch_destroy(b)
         rk.rk_tableset_destroy(ts)
+
+
+def letter_sets(alphabet, n_sets, k, lmin, lmax):
+    rng = np.random.default_rng(n_sets + k)
+    sym = np.frombuffer(alphabet, np.uint8)
+    return [[rng.choice(sym, int(L)).tobytes() for L in rng.integers(lmin, lmax + 1, k)]
+            for _ in range(n_sets)]
+
+
+@pytest.mark.parametrize("alphabet,k,items,total,ctas", [
+    (b"ABCDEFGHIJKLMNOPQRST", 64, 4096, 64 << 20, 3),   # many short texts
+    (b"ABCDEFGHIJKLMNOPQRST", 64, 1024, 1 << 30, 3),    # many chunks
+    (b"ABCDEFGHIJKLMNOPQRST", 64, 1024, 64 << 20, 1),   # few
+    (b"ABCDEFGHIJKLMNOPQRST", 64, 1, 1 << 20, 1),
+    (b"ACGT", 256, 4096, 256 << 20, 1),                 # crowds of survivors
+    (b"ACGT", 256, 4096, 16 << 20, 3),                  # of very short texts
+])
+def test_default_shape(alphabet, k, items, total, ctas):
+    """The launch shape by the limits and the tables, and with it the matches of
+    one text (the texts of a batch may be fewer than its limits)."""
+    pats = letter_sets(alphabet, 3, k, 4, 48)
+    ts = rk.rk_tableset_build(pats)
+    b = rk.rk_batch_create(ts, items, 1 << 20, total, 1 << 20)
+    try:
+        info = rk.rk_batch_info(b)
+        assert info["ctas_per_sm"] == ctas and info["warps"] == (8 if ctas == 3 else 16)
+        rng = np.random.default_rng(k)
+        text = rng.choice(np.frombuffer(alphabet, np.uint8), 150_001)
+        rk.rk_batch_set(b, [1], [to_device(text, 3)], [text.size])
+        rk.rk_batch_run(b)
+        torch.cuda.synchronize()
+        count, status, keys, _ = rk.rk_batch_read(b, 1, 1 << 20)
+        assert status == rk.RK_OK and count <= 1 << 20
+        _, ids, xs = rk.unpack_batch_keys(keys, info["offset_bits"], info["id_bits"])
+        assert_same((ids, xs), oracle.rabin_karp(text, pats[1]), f"{items} {total}")
+    finally:
+        rk.rk_batch_destroy(b)
+        rk.rk_tableset_destroy(ts)
