@@ -344,6 +344,18 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
     const uint32_t mask = (1u << gram_bits) - 1;
     std::vector<uint32_t> gram_at;
     const uint32_t gram_mult = place_prefixes(gram_keys, gram_bits, &gram_at);
+    // Lanes of a warp that compare and lanes that hash wait for each other.  Where a
+    // hash costs about what a comparison does (patterns of at most 8 bytes, prefixes
+    // under 4, so that most windows get here) and many patterns share prefix and
+    // length, all are hashed.  16 MiB, some compared / all hashed: 40 patterns of 1..3
+    // of 20 letters 1370 / 1081 us, of 2..6 of four 1757 / 1347, 200 of 2..4 of
+    // English frequencies 2279 / 1704.
+    uint32_t n_shared = 0;
+    for (const auto &kv : gram_to_lens)
+        for (size_t i = 0; i < kv.second.size(); ++i)
+            n_shared += (i > 0 && kv.second[i - 1].first == kv.second[i].first) ||
+                        (i + 1 < kv.second.size() && kv.second[i + 1].first == kv.second[i].first);
+    const bool hash_all = q < 4 && lmax <= 8 && 3ull * n_shared > k;
     for (uint32_t g = 0; g < D; ++g) {
         const uint32_t key = gram_keys[g];
         const auto &v = gram_to_lens[key];
@@ -353,7 +365,7 @@ int build_blob(const uint8_t *patterns, const uint32_t *lens, uint32_t k, uint32
         for (size_t i = 0; i < v.size();) {
             size_t j = i;
             while (j < v.size() && v[j].first == v[i].first) ++j;
-            const bool one = j == i + 1;
+            const bool one = j == i + 1 && !hash_all;
             const LenRun r{v[i].first, one ? v[i].second : kManyPids,
                            one ? (uint32_t)(poff[v[i].second] / 8) : 0u, 0};
             gram_runs.push_back(r);

@@ -104,6 +104,26 @@ def test_every_density_of_the_prefix_map(opts, lmin, lmax, counts):
         assert_same(gpu_search(pats, text, 5, **opts), expect, f"in the scan, {k}")
 
 
+@pytest.mark.parametrize("alphabet,k,lmin,lmax", [
+    (b"ABCDEFGHIJKLMNOPQRST", 40, 1, 3), (b"ACGT", 40, 2, 6), (b"ACGT", 40, 1, 1),
+    (b"etaoinshr ", 200, 2, 4), (b"ACGT", 8, 1, 2), (b"ACGT", 60, 3, 8), (b"ACGT", 60, 3, 9),
+])
+def test_short_patterns_of_shared_prefixes(alphabet, k, lmin, lmax):
+    """Many patterns of one prefix and length, repeated ones among them, beside
+    prefixes with one."""
+    rng = np.random.default_rng(k + lmax)
+    sym = np.frombuffer(alphabet, np.uint8)
+    text = rng.choice(sym, 50_003)
+    pats = [rng.choice(sym, int(L)).tobytes() for L in rng.integers(lmin, lmax + 1, k)]
+    pats.append(pats[0])
+    expect = oracle.rabin_karp(text, pats)
+    for opts in (dict(), dict(base_log2=1), dict(tile_bytes=1024, stages=2, warps=2)):
+        got, listed = listed_scan(pats, text, 5, **opts)
+        assert_same(got, expect, f"listed {opts}")
+        assert listed > 0
+        assert_same(gpu_search(pats, text, 5, **opts), expect, f"in the scan {opts}")
+
+
 # ---- the tests of the deferred, sampled and role-filter scans, always listed ----
 
 @pytest.fixture
