@@ -269,18 +269,23 @@ __device__ __forceinline__ bool gram_applies(const WinCtx &C, const GramSlot &g,
     return ext_ok || (g.count & kGramShort);
 }
 
-// The prefix-map slot whose lengths apply to a window whose bytes 0..7 are v:
-// exact prefix and gram_applies; -1 if none.
-__device__ __forceinline__ int gram_lookup_v8(const WinCtx &C, uint64_t v) {
+// The prefix-map slot (its content in g) whose lengths apply to a window whose
+// bytes 0..7 are v: exact prefix and gram_applies; -1 if none.
+__device__ __forceinline__ int gram_find(const WinCtx &C, uint64_t v, GramSlot &g) {
     const uint32_t key = C.q == 4 ? (uint32_t)v : (uint32_t)v & ((1u << (8u * C.q)) - 1u);
     const uint32_t gmask = (1u << C.gram_bits) - 1u;
     uint32_t idx = (key * C.gram_mult) >> (32u - C.gram_bits);
     for (;;) {
-        const GramSlot g = C.s2.grams[idx];
+        g = C.s2.grams[idx];
         if (g.count == 0) return -1;
         if (g.key == key) return gram_applies(C, g, v) ? (int)idx : -1;
         idx = (idx + 1) & gmask;
     }
+}
+
+__device__ __forceinline__ int gram_lookup_v8(const WinCtx &C, uint64_t v) {
+    GramSlot g;
+    return gram_find(C, v, g);
 }
 
 template <class Src, class Pos>
@@ -291,16 +296,15 @@ __device__ __forceinline__ int gram_lookup(const WinCtx &C, const Src &src, Pos 
     return gram_lookup_v8(C, v);
 }
 
-// Complete the candidate of prefix-map slot gi at window pos (text offset x):
-// every run that applies, by one comparison (A4), or, where several patterns
+// Complete the candidate of prefix-map slot g at window pos (text offset x, bytes
+// 0..7 v): every run that applies, by one comparison (A4), or, where several patterns
 // share prefix and length, by hash, probe and comparisons (A2, A3, A4); matches
 // emitted (A5).
 template <bool DIRECT = false, class Src, class Pos>
-__device__ __forceinline__ void probe_slot(const WinCtx &C, const WarpCtx &w, const Src &src,
-                                           Pos pos, uint64_t x, uint32_t gi,
+__device__ __forceinline__ void probe_runs(const WinCtx &C, const WarpCtx &w, const Src &src,
+                                           Pos pos, uint64_t x, const GramSlot &g, uint64_t v,
                                            uint32_t cls = kLenAll) {
-    const GramSlot g = C.s2.grams[gi];
-    const bool ext_ok = (g.ext >> ext_bit((uint32_t)(ld8(src, pos) >> (8u * C.q)))) & 1u;
+    const bool ext_ok = (g.ext >> ext_bit((uint32_t)(v >> (8u * C.q)))) & 1u;
     const uint32_t cnt = g.count & ~kGramShort;
     for (uint32_t j = 0; j < cnt; ++j) {
         const LenRun r = C.s2.gram_runs[g.first + j];
@@ -310,6 +314,14 @@ __device__ __forceinline__ void probe_slot(const WinCtx &C, const WarpCtx &w, co
         if (r.pid != kManyPids) compare_one<DIRECT>(C, w, src, pos, x, r);
         else probe_length<DIRECT>(C, w, src, pos, x, r.len);
     }
+}
+
+template <bool DIRECT = false, class Src, class Pos>
+__device__ __forceinline__ void probe_slot(const WinCtx &C, const WarpCtx &w, const Src &src,
+                                           Pos pos, uint64_t x, uint32_t gi,
+                                           uint32_t cls = kLenAll) {
+    const GramSlot g = C.s2.grams[gi];
+    probe_runs<DIRECT>(C, w, src, pos, x, g, ld8(src, pos), cls);
 }
 
 // Every stage after the first for one window at buffer position pos of the
@@ -329,9 +341,9 @@ __device__ __forceinline__ void process_window(const WinCtx &C, const WarpCtx &w
         }
         return;
     }
-    uint64_t v8;
-    const int gi = gram_lookup(C, buf, pos, &v8);
-    if (gi >= 0) probe_slot(C, w, buf, pos, x, (uint32_t)gi);
+    const uint64_t v = ld8(buf, pos);
+    GramSlot g;
+    if (gram_find(C, v, g) >= 0) probe_runs(C, w, buf, pos, x, g, v);
 }
 
 // A candidate for which the list has no room is probed at once, with its
