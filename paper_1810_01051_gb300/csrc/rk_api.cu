@@ -32,12 +32,13 @@ int scan_args_ok(const rk_table *t, const uint8_t *d_text, uint64_t n, const uin
 // of padding in 16 keeps the stores of a warp in different banks), and the
 // windows are then written in order, a warp's 32 hashes side by side.
 //
-// One byte read and eight written per window; bound by the integer pipes (two
-// rotations and two reductions mod p per byte: 90 % busy), the writes take half
-// the time.  128 MiB of text, 16-byte windows: 302 us, 4.0 TB/s, with tiles of
-// 128 threads (256: 310 us, 512: 332 us: every thread adds up the warps before
-// its own).  A rolling update per thread over 64 windows of its own, whose
-// writes lie 512 bytes from its neighbour's: 1553 us.
+// One byte read and eight written per window; bound by the ALU pipe (two
+// rotations and two reductions mod p per byte: 91 % busy, FMA 12 %, the
+// shared-memory data pipe 50 %), the writes take half the time.  128 MiB of text,
+// 16-byte windows: 302 us, 4.0 TB/s, with tiles of 128 threads (256: 310 us, 512:
+// 332 us: every thread adds up the warps before its own).  A rolling update per
+// thread over 64 windows of its own, whose writes lie 512 bytes from its
+// neighbour's: 1553 us.
 __host__ __device__ constexpr uint32_t hash_slot(uint32_t i) { return i + (i >> 4); }
 constexpr uint32_t hash_smem(uint32_t threads) { return 8 * (hash_slot(16 * threads) + 1); }
 
@@ -257,7 +258,7 @@ extern "C" int rk_sort_device(const rk_table *t, uint64_t n, uint64_t *d_keys, u
     int rc = check_device(t);
     if (rc) return rc;
     return launch_sort(t, n, d_keys, capacity, d_info, d_workspace, workspace_bytes,
-                       reinterpret_cast<cudaStream_t>(stream));
+                       reinterpret_cast<cudaStream_t>(stream), false, false);
 }
 
 extern "C" int rk_search_device(const rk_table *t, const uint8_t *d_text, uint64_t n,

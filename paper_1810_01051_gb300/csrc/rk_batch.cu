@@ -84,8 +84,9 @@ __host__ __device__ inline BatchLayout batch_layout(uint32_t warps, uint32_t sta
     return L;
 }
 
-// CTAs per SM that the registers allow: three of 9 warps.  (Two of 17 would leave
-// 60 registers a thread, with spills in the first stage.)
+// CTAs per SM: three of 9 warps, at 72 registers a thread, which spills 40..48 bytes
+// where one CTA has none (100..128 registers).  (Two of 17 warps would leave 60
+// registers, with spills in the first stage.)
 constexpr int batch_ctas(int maxw) { return maxw <= 8 ? 3 : 1; }
 
 template <int MODE, bool Q4, int MAXW, bool S2S>

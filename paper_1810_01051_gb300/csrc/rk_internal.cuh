@@ -37,8 +37,7 @@ struct GroupSlot {
 // it, lengths ascending), and `ext`, a 32-bit fingerprint set of the next four
 // bytes (bytes q..q+3) of the patterns with this prefix that are at least
 // q + 4 bytes long; bit 31 of `count` (kGramShort) marks a prefix that also has
-// a shorter pattern.  Run 0 of slot i is gram_runs[i], so it can be read with
-// the slot; run j > 0 is gram_runs[first + j].
+// a shorter pattern.  Run j of the slot is gram_runs[first + j].
 struct alignas(16) GramSlot {
     uint32_t key;
     uint32_t first;
@@ -261,7 +260,7 @@ int launch_scan_opts(const rk_table *t, const uint8_t *d_text, uint64_t n, uint6
                      const CandList *cand = nullptr, ZeroWords zero = {});
 
 // Tables whose survivors can be verified in a second pass: a stage-1 filter
-// and prefix-map slot indices below 2^24.
+// and prefix-map slot indices below 2^22 (what a candidate holds).
 bool can_defer(const rk_table *t);
 
 // Hash, probe and verify every listed candidate of a deferred scan of
@@ -274,10 +273,11 @@ int launch_verify(const rk_table *t, const uint8_t *d_text, uint64_t n, const Ca
 ZeroWords sort_control(const rk_table *t, uint64_t n, uint64_t capacity, void *d_ws);
 ZeroWords sort_control(int sm_count, uint64_t capacity, void *d_ws);
 
-// `cleared`: the words of sort_control are zero already.
+// `cleared`: the words of sort_control are zero already; `distinct`: no two keys
+// are equal, as in every list that a scan of this library makes.
 int launch_sort(const rk_table *t, uint64_t n, uint64_t *d_keys, uint64_t capacity,
                 const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream,
-                bool cleared = false);
+                bool cleared = false, bool distinct = true);
 
 // The bits of a sort's keys that can be non-zero: lo_bits from bit 0 on and,
 // above them, hi_bits from bit hi_shift on.
@@ -290,7 +290,7 @@ struct SortShape {
 // look-back kernel per 8-bit digit.
 int launch_sort_shape(int sm_count, const SortShape &shape, uint64_t *d_keys, uint64_t capacity,
                       const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream,
-                      bool cleared = false);
+                      bool cleared = false, bool distinct = true);
 
 uint64_t sort_workspace_bytes(uint64_t capacity);
 

@@ -390,6 +390,9 @@ __device__ __forceinline__ void sort_one_tile(uint64_t *keys, uint64_t M, const 
 // keys (1 MiB of DNA, one CTA) 37.9 -> 29.6 us.
 constexpr uint32_t kCellMax = 1024;
 constexpr uint32_t kCrowdedMean = 110;
+// Shorter lists are not sampled (1 us of some 35): with two keys to a thread at
+// most, even kCellMax keys to a cell cost about what the passes do.
+constexpr uint32_t kSampledKeys = 1u << 17;
 constexpr uint32_t kOneCellBits = 12;  // cells of the one-CTA sort
 constexpr uint32_t kOneCellMax = 96;   // and the most keys it compares in one
 
@@ -439,12 +442,17 @@ __device__ __forceinline__ uint32_t cta_excl(uint32_t v, uint32_t *wsum, uint32_
 }
 
 // The keys before key k, which lies at tmp[own], in its cell [b, e): the smaller
-// ones, and of equal ones those at lower places (counted again, as only a list
-// that its caller made has any; a test of j < own in the one loop: 5 M keys, 78 to
-// a cell, 397 us, this 340, smaller keys alone 303; 1.2 to a cell 196, 196, 192).
+// ones, and of equal ones those at lower places (counted again, as they are rare;
+// a test of j < own in the one loop: 5 M keys, 97 to a cell, 397 us, this 340,
+// smaller keys alone 303; 1.2 to a cell 196, 196, 192).  Only a list that a caller
+// made has equal keys: the library's own are told to be distinct.
 __device__ __forceinline__ uint32_t place_in_cell(const uint64_t *tmp, uint32_t b, uint32_t e,
-                                                  uint32_t own, uint64_t k) {
+                                                  uint32_t own, uint64_t k, bool distinct) {
     uint32_t less = 0, same = 0;
+    if (distinct) {
+        for (uint32_t j = b; j < e; ++j) less += tmp[j] < k;
+        return less;
+    }
     for (uint32_t j = b; j < e; ++j) {
         const uint64_t v = tmp[j];
         less += v < k;
@@ -459,7 +467,8 @@ __device__ __forceinline__ uint32_t place_in_cell(const uint64_t *tmp, uint32_t 
 // with the keys untouched, when a cell holds too many or a key is outside the
 // shape.
 __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const SortShape &shape,
-                                               uint64_t *sbuf, uint32_t *cell, uint32_t *wsum) {
+                                               uint64_t *sbuf, uint32_t *cell, uint32_t *wsum,
+                                               bool distinct) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr uint32_t kCells = 1u << kOneCellBits, kPer = kCells / kThreads;
     constexpr uint32_t kKeys = kSortTile / kThreads;
@@ -510,7 +519,7 @@ __device__ __forceinline__ bool sort_one_cells(uint64_t *keys, uint32_t M, const
     for (uint32_t r = 0; r < kKeys; ++r)
         if (r * kThreads + tid < M) {
             const uint32_t b = cell[cr[r] >> 16], e = cell[(cr[r] >> 16) + 1];
-            keys[b + place_in_cell(sbuf, b, e, b + (cr[r] & 0xFFFFu), key[r])] = key[r];
+            keys[b + place_in_cell(sbuf, b, e, b + (cr[r] & 0xFFFFu), key[r], distinct)] = key[r];
         }
     return true;
 }
@@ -560,7 +569,8 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
                                                   uint16_t *rank, uint32_t *part, uint32_t cb,
                                                   uint32_t *flag, unsigned int *bar, uint32_t G,
                                                   unsigned int *passed, unsigned long long *info,
-                                                  uint32_t *seen, uint32_t *wsum, int *s_ok) {
+                                                  uint32_t *seen, uint32_t *wsum, int *s_ok,
+                                                  bool distinct) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t C = 1u << cb;
     const uint32_t tb = shape.lo_bits + shape.hi_bits;
@@ -571,16 +581,21 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
 
     // a CTA's samples are spread over the whole list: neighbours in it come from
     // one stretch of text, so a run of them would look crowded
-    const uint64_t sample =
-        __ldcg(keys + ((uint64_t)tid * G + blockIdx.x) * M / ((uint64_t)kThreads * G));
-    for (uint32_t i = tid; i < kSeen; i += kThreads) seen[i] = 0;
+    const bool sampled = M > kSampledKeys;
+    uint64_t sample = 0;
+    if (sampled) {
+        sample = __ldcg(keys + ((uint64_t)tid * G + blockIdx.x) * M / ((uint64_t)kThreads * G));
+        for (uint32_t i = tid; i < kSeen; i += kThreads) seen[i] = 0;
+    }
     for (uint64_t i = gid; i < C / 4; i += stride)
         __stcg(reinterpret_cast<uint4 *>(cnt) + i, make_uint4(0, 0, 0, 0));
-    const uint32_t pairs = sample_pairs(sample, shape, cs, outside, seen, wsum, lane, warp);
-    if (tid == 0 && pairs) atomicAdd(flag + 1, pairs);
+    if (sampled) {
+        const uint32_t pairs = sample_pairs(sample, shape, cs, outside, seen, wsum, lane, warp);
+        if (tid == 0 && pairs) atomicAdd(flag + 1, pairs);
+    }
     if (!grid_sync(bar, ++*passed * G, info, s_ok)) return kCellsTimeout;
     // two keys share a cell with a chance of (mean size - 1) / M
-    if ((uint64_t)__ldcg(flag + 1) * M >
+    if (sampled && (uint64_t)__ldcg(flag + 1) * M >
         (uint64_t)G * (kThreads * (kThreads - 1) / 2) * (kCrowdedMean - 1))
         return kCellsCrowded;
 
@@ -680,7 +695,7 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
         for (uint32_t u = 0; u < kV; ++u)
             if (i0 + u * stride < M) {
                 const uint32_t own = (uint32_t)(i0 + u * stride);
-                keys[b[u] + place_in_cell(tmp, b[u], e[u], own, k[u])] = k[u];
+                keys[b[u] + place_in_cell(tmp, b[u], e[u], own, k[u], distinct)] = k[u];
             }
     }
     return kCellsDone;
@@ -706,7 +721,7 @@ __device__ __forceinline__ CellsResult sort_cells(uint64_t *keys, uint64_t *tmp,
 __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
     uint64_t *keys, uint64_t *tmp, unsigned long long *info, uint64_t cap, Shifts sh,
     SortShape shape, uint32_t *cnt, uint64_t cnt_bytes, uint32_t pitch, uint32_t *totals,
-    unsigned int *bar, uint32_t *flag) {
+    unsigned int *bar, uint32_t *flag, bool distinct) {
     uint64_t M;
     uint32_t T;
     if (!sort_count(info, cap, &M, &T)) return;
@@ -722,7 +737,7 @@ __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
     if (T == 1) {
         __shared__ uint64_t sbuf[kSortTile];
         __shared__ __align__(16) uint32_t cell[(1u << kOneCellBits) + 4];
-        if (!sort_one_cells(keys, (uint32_t)M, shape, sbuf, cell, wsum))
+        if (!sort_one_cells(keys, (uint32_t)M, shape, sbuf, cell, wsum, distinct))
             sort_one_tile(keys, M, sh, sbuf, wcnt, dbase, wsum);
         return;
     }
@@ -736,7 +751,7 @@ __global__ void __launch_bounds__(kThreads) rk_sort_fused_kernel(
         uint16_t *rank = reinterpret_cast<uint16_t *>(cnt + (1u << cb) + 4);
         uint32_t *part = reinterpret_cast<uint32_t *>(rank + (M + 1) / 2 * 2);
         const CellsResult r = sort_cells(keys, tmp, M, shape, cnt, rank, part, cb, flag, bar, G,
-                                         &passed, info, &wcnt[0][0], wsum, &s_ok);
+                                         &passed, info, &wcnt[0][0], wsum, &s_ok, distinct);
         if (r != kCellsCrowded) return;
     }
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -915,7 +930,7 @@ uint64_t sort_workspace_bytes(uint64_t capacity) { return sort_ws_bytes(capacity
 
 int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
                       uint64_t capacity, const uint64_t *d_info, void *d_ws, uint64_t ws_bytes,
-                      cudaStream_t stream, bool cleared) {
+                      cudaStream_t stream, bool cleared, bool distinct) {
     SortShape shape = shape_in;
     Shifts sh = shifts_of(shape);
     if (capacity < 2 || sh.n == 0) return RK_OK;
@@ -943,7 +958,7 @@ int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
         unsigned int *bar = counters + 32;
         uint32_t *flag = counters;
         void *args[] = {&d_keys, &tmp,       &info,  &capacity, &sh,  &shape,
-                        &cnt,    &cnt_bytes, &pitch, &totals,   &bar, &flag};
+                        &cnt,    &cnt_bytes, &pitch, &totals,   &bar, &flag, &distinct};
         if (cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(rk_sort_fused_kernel), g,
                                         kThreads, args, 0, stream) != cudaSuccess) {
             cudaGetLastError();
@@ -975,10 +990,10 @@ int launch_sort_shape(int sm_count, const SortShape &shape_in, uint64_t *d_keys,
 
 int launch_sort(const rk_table *t, uint64_t n, uint64_t *d_keys, uint64_t capacity,
                 const uint64_t *d_info, void *d_ws, uint64_t ws_bytes, cudaStream_t stream,
-                bool cleared) {
+                bool cleared, bool distinct) {
     if (n == 0 || t->dev.n_patterns == 0) return RK_OK;
     return launch_sort_shape(t->sm_count, plain_shape(n, t->dev.n_patterns), d_keys, capacity,
-                             d_info, d_ws, ws_bytes, stream, cleared);
+                             d_info, d_ws, ws_bytes, stream, cleared, distinct);
 }
 
 ZeroWords sort_control(int sm_count, uint64_t capacity, void *d_ws) {
