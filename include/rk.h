@@ -311,7 +311,7 @@ int rk_search_device_matches(const rk_table *t, const uint8_t *d_text, uint64_t 
 void rk_free_matches(rk_match *m);
 
 /* Rabin hash of every length-L window (Section 3.1's hash h = h*B + c,
- * reduced mod 2^61-1, B = 2^base_log2), by a tiled rolling update:
+ * reduced mod 2^61-1, B = 2^base_log2), from the prefix hashes of a tile:
  *   d_hashes[x] = sum_{i<L} d_text[x+i] * B^(L-1-i)  mod (2^61 - 1),
  *   x = 0 .. n-L  (nothing is written when L > n).
  * L in 1..RK_MAX_PATTERN_LEN, base_log2 in 1..60.  Errors: RK_EINVAL, RK_ECUDA. */
